@@ -717,8 +717,8 @@ int reed_run(reed_ctx* ctx, double ion_Z, double ion_M, double energy_eV, double
         P.adj_every = every;
         P.adj_nck = seg / every + 1;
     }
-    const size_t smem = f64 ? reed_f64::smem_bytes(tt, P.na, P.bond_cap, P.adjoint, P.g_nbins, P.act_cap)
-                            : reed_f32::smem_bytes(tt, P.na, P.bond_cap, P.adjoint, P.g_nbins, P.act_cap);
+    const size_t smem = f64 ? reed_f64::track_smem_bytes(tt, P.na, P.bond_cap, P.adjoint, P.g_nbins, P.act_cap)
+                            : reed_f32::track_smem_bytes(tt, P.na, P.bond_cap, P.adjoint, P.g_nbins, P.act_cap);
     if (smem > ctx->smem_optin)
         return fail(ctx, REED_E_SMEM, "window of %d atoms needs %zu B of shared memory (max %zu)", P.na, smem,
                     ctx->smem_optin);
@@ -1593,8 +1593,8 @@ extern "C" int reed_run_static(const reed_lattice* lat, const reed_species* sp, 
 
     const int tt = P.tt;
     const bool f64 = o.precision == REED_PREC_FP64;
-    const size_t smem = f64 ? reed_f64::smem_bytes(tt, P.na, P.bond_cap, 0, P.g_nbins, P.act_cap)
-                            : reed_f32::smem_bytes(tt, P.na, P.bond_cap, 0, P.g_nbins, P.act_cap);
+    const size_t smem = f64 ? reed_f64::track_smem_bytes(tt, P.na, P.bond_cap, 0, P.g_nbins, P.act_cap)
+                            : reed_f32::track_smem_bytes(tt, P.na, P.bond_cap, 0, P.g_nbins, P.act_cap);
     if (smem > (size_t)optin)
         return fail(nullptr, REED_E_SMEM, "window of %d atoms needs %zu B of shared memory (max %d)", P.na, smem, optin);
     LaunchCfg L;

@@ -15,6 +15,7 @@ struct LaunchCfg {
 // Per-precision launchers (prec: REED_PREC_MIXED -> float, REED_PREC_FP64 -> double).
 namespace reed_f32 {
 size_t smem_bytes(int tt, int na, int bond_cap, int adj = 0, int nbins = 0, int act = 0);
+size_t track_smem_bytes(int tt, int na, int bond_cap, int adj, int nbins, int act);
 size_t spill_bytes(int tt);
 size_t adj_scratch_bytes(const DevParams& P, size_t entry);
 size_t entry_bytes(int tt, int na);
@@ -30,6 +31,7 @@ cudaError_t launch_cell_atoms(const DevParams& P, uint64_t key, int ix, int iy, 
 }  // namespace reed_f32
 namespace reed_f64 {
 size_t smem_bytes(int tt, int na, int bond_cap, int adj = 0, int nbins = 0, int act = 0);
+size_t track_smem_bytes(int tt, int na, int bond_cap, int adj, int nbins, int act);
 size_t spill_bytes(int tt);
 size_t adj_scratch_bytes(const DevParams& P, size_t entry);
 size_t entry_bytes(int tt, int na);

@@ -64,7 +64,7 @@ __device__ __forceinline__ R ion_pair(const HotParams<R>& H, int spline_on, int 
     const R ir = Mth<R>::rsqrt(r2);
     const R r = r2 * ir;
     R V, dV;
-    Zbl<R>::eval(r, ir, H.zk[s], H.zia[s], V, dV);
+    Zbl<R>::eval(r, ir, s ? H.zk[1] : H.zk[0], s ? H.zia[1] : H.zia[0], V, dV);
     if (spline_on) {
         const R lr = Mth<R>::log(r);
         R c = R(0), dc = R(0);

@@ -33,7 +33,13 @@
 enum { SRC_NONE = 0, SRC_PRIMARY = 1, SRC_CLONE = 2, SRC_STOLEN = 3 };
 enum { POOL_EMPTY = 0, POOL_WRITING = 1, POOL_FULL = 2, POOL_READING = 3 };
 
-enum { EV_NONE = 0, EV_END = 1, EV_CLONE = 2, EV_CKPT = 3 };
+enum { EV_NONE = 0, EV_END = 1, EV_CLONE = 2 };
+
+// counters a CTA of the ion-target-only model keeps in shared memory
+enum {
+    ION_PRIM = 0, ION_CLONES, ION_TRACKS, ION_STEPS, ION_PAIRS, ION_SHIFTS, ION_DROPS, ION_FAILS, ION_MOVED, ION_PH_ION,
+    ION_PH_FORCE, ION_PH_ADMIN, ION_NCOUNT
+};
 
 // Ion state as stored in shared memory and in clone records.  Position,
 // time and the energy given to electronic stopping are FP64 accumulators;
@@ -68,6 +74,8 @@ template <typename R> struct TrackShared {
     int Aold[3];
     int shift, event, status, src, top, nclone, slot;
     int need_count, active_count;
+    int nhit0;            // ion-target-only model: atoms within the cutoff at the last list build
+    unsigned long long cnt[ION_NCOUNT];   // ion-target-only model: counters of this CTA, flushed at exit
     int nspill;           // overflow rows taken by the current lists
     int ncls[4];          // Tersoff: slots per centre-pass class, in `order` (see ters_centres)
     unsigned long long cls_sum[4];   // centre evaluations per class, summed over passes (thread 0)
@@ -1558,43 +1566,6 @@ struct WorkCount {
 // Writes W.frc of every present atom.  With target-target terms the
 // integrated atoms are visited through their list slots (balanced across
 // threads); the others only contribute ion-target pairs.
-// The ion-target part of one atom's force pass at its current position p,
-// and (integrated atoms) the second half kick: the operations of atom_force
-// for an atom without target-target terms, on values held in registers.
-template <typename R>
-__device__ __forceinline__ void ion_atom_step(const DevParams& P, const HotParams<R>& H, const TrackShared<R>* S,
-                                              const V4<R>& p, V4<R>& v, bool act, R hdt, V4<R>& f, Partial<R>& out)
-{
-    R fx = R(0), fy = R(0), fz = R(0);
-    const R dx = p.x - S->rel[0], dy = p.y - S->rel[1], dz = p.z - S->rel[2];
-    const R r2 = dx * dx + dy * dy + dz * dz;
-    if (r2 < H.rc2) {
-        R U, rw;
-        const R g = ion_pair<R>(H, P.spline_on, P.rho_on, species_of(p), r2, U, rw);
-        fx -= g * dx;
-        fy -= g * dy;
-        fz -= g * dz;
-        out.fx += g * dx;
-        out.fy += g * dy;
-        out.fz += g * dz;
-        out.rho += rw;
-        out.epot += U;
-        out.pairs += 1;
-    }
-    f.x = fx;
-    f.y = fy;
-    f.z = fz;
-    f.w = R(0);
-    if (act) {
-        const R kk = hdt * H.invM2[species_of(p)];
-        v.x += kk * fx;
-        v.y += kk * fy;
-        v.z += kk * fz;
-        out.vmax2 = max(out.vmax2, v.x * v.x + v.y * v.y + v.z * v.z);
-        if (H.de_max > R(0)) out.pmax = max(out.pmax, fabs(fx * v.x + fy * v.y + fz * v.z));
-    }
-}
-
 template <typename R, int TT, bool KICK>
 __device__ __forceinline__ void atom_force(const DevParams& P, const HotParams<R>& H, Win<R, TT>& W, int i, int k,
                                            R hdt, Partial<R>& out, bool want_energy)
@@ -1788,16 +1759,20 @@ __device__ long long finish_track(const DevParams& P, const DevBuf& B, const Ion
 // on an MeV ion over its 0.05 A steps -- do not round systematically: with a
 // plain FP32 sum the 85 MeV Kr drag-only range came out 0.7 % short, with the
 // two-float sum within 1e-6.
-template <typename R> __device__ __forceinline__ void add_velocity(IonState<R>& I, int d, R inc)
+template <typename R> __device__ __forceinline__ void add_velocity(R& v, R& vlo, R inc)
 {
     if constexpr (sizeof(R) == 4) {
-        const float a = I.v[d], b = __fadd_rn(inc, I.vlo[d]);
+        const float a = v, b = __fadd_rn(inc, vlo);
         const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-        I.vlo[d] = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-        I.v[d] = s;
+        vlo = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+        v = s;
     } else {
-        I.v[d] += inc;
+        v += inc;
     }
+}
+template <typename R> __device__ __forceinline__ void add_velocity(IonState<R>& I, int d, R inc)
+{
+    add_velocity<R>(I.v[d], I.vlo[d], inc);
 }
 
 // Launch a primary (Sec. 2; lateral position uniform in the (0,0) surface
@@ -2025,12 +2000,10 @@ template <typename R, int TT>
 __device__ void initial_forces(const DevParams& P, const HotParams<R>& H, Win<R, TT>& W, unsigned long long& ctr_bonds,
                                unsigned long long& ctr_rebuild, int& nbovf, int& capovf, WorkCount& wc)
 {
-    if constexpr (TT != REED_TT_NONE) {
-        build_neighbours<R, TT>(P, H, W, nbovf, capovf, wc.spilled);
-        if (threadIdx.x == 0) ++ctr_rebuild;
-        __syncthreads();
-        if (P.nl_check) check_lists<R, TT>(P, H, W, H.rlist2, wc.nl_errors);
-    }
+    build_neighbours<R, TT>(P, H, W, nbovf, capovf, wc.spilled);
+    if (threadIdx.x == 0) ++ctr_rebuild;
+    __syncthreads();
+    if (P.nl_check) check_lists<R, TT>(P, H, W, H.rlist2, wc.nl_errors);
     if constexpr (TT == REED_TT_TERSOFF) {
         ters_centres<R, TT>(H, W, wc.triplets);
         __syncthreads();
@@ -2055,34 +2028,28 @@ __device__ void initial_forces(const DevParams& P, const HotParams<R>& H, Win<R,
 #include "reed_adjoint.cuh"
 
 // ---------------------------------------------------------------------------
-// The persistent kernel.  ADJ (target model NONE only) adds the checkpoints,
-// the step records and the reverse pass of the truncated-segment adjoint.
+// The persistent kernel of the models with target-target forces (the
+// ion-target-only model and its adjoint: reed_ion.cuh).
 // The second launch bound is the number of CTAs per SM the shared memory of
 // the workloads allows, so registers are budgeted for that occupancy.
 // ---------------------------------------------------------------------------
-template <typename R, int TT, bool ADJ>
-constexpr int track_min_ctas()
-{
-    if (TT == REED_TT_NONE) return sizeof(R) == 4 ? (ADJ ? 2 : 3) : (ADJ ? 1 : 2);
-    return TT == REED_TT_TERSOFF && sizeof(R) == 4 ? 2 : 1;
-}
+template <typename R, int TT> constexpr int track_min_ctas() { return TT == REED_TT_TERSOFF && sizeof(R) == 4 ? 2 : 1; }
 
 // Threads per track at most: 512 for the pair-list model (one track fills an
 // SM's shared memory, so its warps are all the SM gets), else 256.
 template <int TT> constexpr int track_max_threads() { return TT == REED_TT_BUCKINGHAM ? 512 : 256; }
 
-template <typename R, int TT, bool ADJ>
-__global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, TT, ADJ>())) reed_track_kernel(
+template <typename R, int TT>
+__global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, TT>())) reed_track_kernel(
     const __grid_constant__ DevParams P, const __grid_constant__ DevBuf B)
 {
-    static_assert(!ADJ || TT == REED_TT_NONE, "the adjoint runs without target-target forces");
+    static_assert(TT != REED_TT_NONE, "the ion-target-only model has its own kernel");
     extern __shared__ __align__(16) unsigned char smem[];
-    Win<R, TT> W(smem, P.na, P.bond_cap, ADJ ? 1 : 0, P.g_nbins, P.act_cap,
+    Win<R, TT> W(smem, P.na, P.bond_cap, 0, P.g_nbins, P.act_cap,
                  B.spill ? B.spill + (size_t)blockIdx.x * B.spill_stride : nullptr);
     TrackShared<R>* S = W.S;
     const HotParams<R>& H = hot<R>(P);
     const int tid = threadIdx.x;
-    unsigned char* adjbase = (ADJ && B.adj) ? B.adj + (size_t)blockIdx.x * B.adj_stride : nullptr;
     unsigned char* stack = B.stacks ? B.stacks + (size_t)blockIdx.x * B.stack_stride : nullptr;
 
     // thread-0 counters, flushed at exit
@@ -2171,12 +2138,6 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
             }
             __syncthreads();
             initial_forces<R, TT>(P, H, W, c_bonds, c_rebuild, nbovf, capovf, wc);
-            if constexpr (TT == REED_TT_NONE) {
-                if (ADJ && adjbase) {   // checkpoint of the state before step 0
-                    save_state<R, TT>(P, W, adjbase);
-                    __syncthreads();
-                }
-            }
         } else if (src == SRC_STOLEN) {
             const unsigned char* rec = B.pool + (size_t)S->slot * B.entry_bytes;
             if (tid == 0) {
@@ -2194,10 +2155,8 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
                 atomicSub(&B.pool_ctl[1], 1u);
                 if (B.splits) atomicAdd(&B.splits[REED_MAX_THR], 1ull);
             }
-            if constexpr (TT != REED_TT_NONE) {
-                build_neighbours<R, TT>(P, H, W, nbovf, capovf, wc.spilled);
-                if (tid == 0) ++c_rebuild;
-            }
+            build_neighbours<R, TT>(P, H, W, nbovf, capovf, wc.spilled);
+            if (tid == 0) ++c_rebuild;
             __syncthreads();
         } else {
             unsigned char* rec = stack + (size_t)(S->top - 1) * B.entry_bytes;
@@ -2208,10 +2167,8 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
             copy_window<R, TT>(P, W, rec, false);
             __syncthreads();
             if (tid == 0) S->top -= 1;
-            if constexpr (TT != REED_TT_NONE) {
-                build_neighbours<R, TT>(P, H, W, nbovf, capovf, wc.spilled);
-                if (tid == 0) ++c_rebuild;
-            }
+            build_neighbours<R, TT>(P, H, W, nbovf, capovf, wc.spilled);
+            if (tid == 0) ++c_rebuild;
             __syncthreads();
         }
         const bool tracing = (src == SRC_PRIMARY) && (S->pidx < P.trace_tracks);
@@ -2230,48 +2187,6 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
             const int shift = S->shift;
             const uint64_t key = S->ion.key;
             Partial<R> q = {R(0), R(0), R(0), R(0), R(0), R(0), 0, 0};
-            if constexpr (TT == REED_TT_NONE) {
-                // no target-target forces: each atom's whole step (re-anchor,
-                // half kick, drift, ion-target force, half kick) in one pass,
-                // the same operations as the separate phases of the other models
-                for (int i = tid; i < P.na; i += blockDim.x) {
-                    V4<R> p = W.pos[i], v = W.vel[i], f = W.frc[i];
-                    // half kick and drift of the atoms integrated before the
-                    // window moves, then the move (a step's kick and drift
-                    // precede its window update)
-                    if (is_active(p)) {
-                        ++wc.moved;
-                        const R k = hdt * H.invM2[species_of(p)];
-                        v.x += k * f.x;
-                        v.y += k * f.y;
-                        v.z += k * f.z;
-                        p.x += dt * v.x;
-                        p.y += dt * v.y;
-                        p.z += dt * v.z;
-                    }
-                    if (shift) {
-                        const V4<R> p0 = p, v0 = v;
-                        if (reanchor_atom<R>(P, H, key, i, S->Aold, S->ion.A, p, v, f))
-                            deposit_damage<R>(P, B, p0, v0, S->Aold, ldexp(1.0, -S->ion.level));
-                    }
-                    if (!is_present(p)) {
-                        if (shift) {
-                            W.pos[i] = p;
-                            W.vel[i] = v;
-                            W.frc[i] = f;
-                        }
-                        continue;
-                    }
-                    const bool act = is_active(p);
-                    ion_atom_step<R>(P, H, W.S, p, v, act, hdt, f, q);
-                    W.pos[i] = p;
-                    W.vel[i] = v;
-                    W.frc[i] = f;
-                }
-                reduce_partials<R, TT>(W, q);
-                __syncthreads();
-                lap(PH_FORCE);
-            } else {
             // phase A: first half kick + drift of the atoms integrated before
             // the window moves, then the move (a step's kick and drift precede
             // its window update: an atom entering the integrated region is
@@ -2293,14 +2208,13 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
                     p.x += sx;
                     p.y += sy;
                     p.z += sz;
-                    if constexpr (TT != REED_TT_NONE) {
-                        { const R l2 = sx * sx + sy * sy + sz * sz; if (l2 > R(0)) v.w += l2 * Mth<R>::rsqrt(l2); }
-                        if (v.w > pm1) {
-                            pm2 = pm1;
-                            pm1 = v.w;
-                        } else if (v.w > pm2) {
-                            pm2 = v.w;
-                        }
+                    const R l2 = sx * sx + sy * sy + sz * sz;
+                    if (l2 > R(0)) v.w += l2 * Mth<R>::rsqrt(l2);
+                    if (v.w > pm1) {
+                        pm2 = pm1;
+                        pm1 = v.w;
+                    } else if (v.w > pm2) {
+                        pm2 = v.w;
                     }
                 }
                 if (shift) {
@@ -2312,51 +2226,48 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
                 W.vel[i] = v;
                 if (shift) W.frc[i] = f;
             }
-            if constexpr (TT != REED_TT_NONE) {
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const R q1 = __shfl_xor_sync(0xffffffffu, pm1, o), q2 = __shfl_xor_sync(0xffffffffu, pm2, o);
-                    pm2 = fmax(fmin(pm1, q1), fmax(pm2, q2));
-                    pm1 = fmax(pm1, q1);
-                }
-                if ((tid & 31) == 0) {
-                    S->path2[tid >> 5][0] = pm1;
-                    S->path2[tid >> 5][1] = pm2;
-                }
-                __syncthreads();
-                lap(PH_MOVE);
-                // every thread merges the per-warp pairs in the same order
-                R m1 = R(0), m2 = R(0);
-                for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-                    const R q1 = S->path2[w][0], q2 = S->path2[w][1];
-                    m2 = fmax(fmin(m1, q1), fmax(m2, q2));
-                    m1 = fmax(m1, q1);
-                }
-                if (shift || m1 + m2 > H.skin) {
-                    bool refreshed = false;
-                    if constexpr (TT == REED_TT_TERSOFF) {
-                        if (!shift) refreshed = refresh_lists<R, TT>(P, H, W, nbovf, wc.spilled);
-                    }
-                    if (!refreshed) build_neighbours<R, TT>(P, H, W, nbovf, capovf, wc.spilled);
-                    __syncthreads();
-                    if (tid == 0) ++(refreshed ? wc.refreshes : c_rebuild);
-                    if (P.nl_check)
-                        check_lists<R, TT>(P, H, W, refreshed ? H.tcut * H.tcut : H.rlist2, wc.nl_errors);
-                    lap(PH_BUILD);
-                }
+            for (int o = 16; o > 0; o >>= 1) {
+                const R q1 = __shfl_xor_sync(0xffffffffu, pm1, o), q2 = __shfl_xor_sync(0xffffffffu, pm2, o);
+                pm2 = fmax(fmin(pm1, q1), fmax(pm2, q2));
+                pm1 = fmax(pm1, q1);
+            }
+            if ((tid & 31) == 0) {
+                S->path2[tid >> 5][0] = pm1;
+                S->path2[tid >> 5][1] = pm2;
+            }
+            __syncthreads();
+            lap(PH_MOVE);
+            // every thread merges the per-warp pairs in the same order
+            R m1 = R(0), m2 = R(0);
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+                const R q1 = S->path2[w][0], q2 = S->path2[w][1];
+                m2 = fmax(fmin(m1, q1), fmax(m2, q2));
+                m1 = fmax(m1, q1);
+            }
+            if (shift || m1 + m2 > H.skin) {
+                bool refreshed = false;
                 if constexpr (TT == REED_TT_TERSOFF) {
-                    ters_centres<R, TT>(H, W, wc.triplets);
-                    __syncthreads();
-                    lap(PH_PASS1);
-                    if (tid == 0)
-                        for (int c = 0; c < 4; ++c) S->cls_sum[c] += (unsigned)S->ncls[c];
+                    if (!shift) refreshed = refresh_lists<R, TT>(P, H, W, nbovf, wc.spilled);
                 }
+                if (!refreshed) build_neighbours<R, TT>(P, H, W, nbovf, capovf, wc.spilled);
+                __syncthreads();
+                if (tid == 0) ++(refreshed ? wc.refreshes : c_rebuild);
+                if (P.nl_check)
+                    check_lists<R, TT>(P, H, W, refreshed ? H.tcut * H.tcut : H.rlist2, wc.nl_errors);
+                lap(PH_BUILD);
+            }
+            if constexpr (TT == REED_TT_TERSOFF) {
+                ters_centres<R, TT>(H, W, wc.triplets);
+                __syncthreads();
+                lap(PH_PASS1);
+                if (tid == 0)
+                    for (int c = 0; c < 4; ++c) S->cls_sum[c] += (unsigned)S->ncls[c];
             }
             force_phase<R, TT, true>(P, H, W, hdt, q, false);
             reduce_partials<R, TT>(W, q);
             __syncthreads();
             lap(PH_FORCE);
-            }
             if (tid == 0) {
                 R red[REED_NRED];
                 gather_partials<R, TT>(W, red);
@@ -2374,18 +2285,6 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
                     int* a3 = B.trace_anchor + 3 * o;
                     a3[0] = I.A[0]; a3[1] = I.A[1]; a3[2] = I.A[2];
                 }
-                if (adjbase) {
-                    // frozen quantities of this step; checkpoints every adj_every steps
-                    StepRec<R>* ring = reinterpret_cast<StepRec<R>*>(adjbase + (size_t)P.adj_nck * B.entry_bytes);
-                    StepRec<R> sr;
-                    sr.dt = S->dt;
-                    sr.A[0] = S->ion.A[0];
-                    sr.A[1] = S->ion.A[1];
-                    sr.A[2] = S->ion.A[2];
-                    sr.flags = (S->on1 ? 1 : 0) | (S->on2 ? 2 : 0) | (shift ? 4 : 0);
-                    ring[(S->ion.steps - 1) % REED_STEP_RING] = sr;
-                    if (ev == EV_NONE && S->ion.steps % P.adj_every == 0) ev = EV_CKPT;
-                }
                 S->event = ev;
                 if (ev == EV_NONE) ion_prologue<R>(P, H, S);
             }
@@ -2398,13 +2297,6 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
             }
             need_prologue = true;
             if (ev == EV_END) break;
-            if (ev == EV_CKPT) {
-                if constexpr (TT == REED_TT_NONE) {
-                    save_state<R, TT>(P, W, adjbase + (size_t)((S->ion.steps / P.adj_every) % P.adj_nck) * B.entry_bytes);
-                    __syncthreads();
-                }
-                continue;
-            }
             // ---- cloning (Sec. 2): push one record per level passed
             const int nc = S->nclone;
             __syncthreads();
@@ -2488,23 +2380,10 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
                 ++c_fail;
                 atomicOr(B.status, ERR_NONFINITE);
             }
-            S->rec_index = finish_track<R>(P, B, S->ion, S->status);
+            finish_track<R>(P, B, S->ion, S->status);
             ++c_tracks;
         }
         __syncthreads();
-        if constexpr (ADJ) {
-            // truncated-segment sensitivities of the final depth
-            if (adjbase && B.grads && S->rec_index >= 0) {
-                double g[REED_NTHETA] = {0, 0, 0, 0, 0, 0, 0, 0};
-                if (S->status == REED_TRACK_STOPPED) {
-                    AdjScratch<R, TT> A(adjbase, P, B.entry_bytes);
-                    adjoint_track<R, TT>(P, H, W, A, g);
-                }
-                if (tid == 0)
-                    for (int k = 0; k < REED_NTHETA; ++k) B.grads[(size_t)S->rec_index * REED_NTHETA + k] = g[k];
-                __syncthreads();
-            }
-        }
     }
     if (nbovf || capovf) atomicOr(B.status, ERR_NEIGHBOR);
     // flush counters
