@@ -267,7 +267,7 @@ __device__ void replay_step(const DevParams& P, const HotParams<R>& H, Win<R, TT
     __syncthreads();
     if (threadIdx.x == 0) {
         R red[REED_NRED];
-        gather_partials<R, TT>(W, red);
+        gather_partials<R, TT>(W, red, (int)blockDim.x >> 5);
         IonState<R>& I = S->ion;
         for (int d = 0; d < 3; ++d) I.f[d] = red[d];
         I.rho = red[3];

@@ -729,8 +729,8 @@ int reed_run(reed_ctx* ctx, double ion_Z, double ion_M, double energy_eV, double
                                     : (tuned ? ctx->tuned_threads[pi][ai] : (tt == REED_TT_NONE ? 64 : 256));
     L.smem = smem;
     int occ = 0;
-    CK(f64 ? reed_f64::occupancy(tt, L.threads, smem, &occ, P.adjoint)
-           : reed_f32::occupancy(tt, L.threads, smem, &occ, P.adjoint));
+    CK(f64 ? reed_f64::occupancy(tt, L.threads, smem, &occ, P.adjoint, P.act_cap)
+           : reed_f32::occupancy(tt, L.threads, smem, &occ, P.adjoint, P.act_cap));
     if (occ < 1) return fail(ctx, REED_E_SMEM, "kernel does not fit on an SM (%zu B shared, %d threads)", smem, L.threads);
     L.ctas_per_sm = o.ctas_per_sm ? std::min(o.ctas_per_sm, occ) : (tuned ? std::min(ctx->tuned_ctas[pi][ai], occ) : occ);
     L.grid = ctx->sms * L.ctas_per_sm;
@@ -1601,8 +1601,8 @@ extern "C" int reed_run_static(const reed_lattice* lat, const reed_species* sp, 
     L.threads = o.threads_per_track ? o.threads_per_track : (tt == REED_TT_NONE ? 64 : 256);
     L.smem = smem;
     int occ = 0;
-    CK(f64 ? reed_f64::occupancy(tt, L.threads, smem, &occ, P.adjoint)
-           : reed_f32::occupancy(tt, L.threads, smem, &occ, P.adjoint));
+    CK(f64 ? reed_f64::occupancy(tt, L.threads, smem, &occ, P.adjoint, P.act_cap)
+           : reed_f32::occupancy(tt, L.threads, smem, &occ, P.adjoint, P.act_cap));
     if (occ < 1) return fail(nullptr, REED_E_SMEM, "kernel does not fit on an SM");
     L.ctas_per_sm = o.ctas_per_sm ? std::min(o.ctas_per_sm, occ) : occ;
 

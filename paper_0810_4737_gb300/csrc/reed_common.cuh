@@ -17,7 +17,8 @@
 
 #define REED_MAX_BASIS 12
 #define REED_MAX_THR 16
-#define REED_MAX_WARPS 16
+#define REED_MAX_WARPS 24       // warps of a track's CTA at most (768 threads: one per atom of a 4^3-cell CeO2 window)
+#define REED_ADJ_WARPS 8        // ... of an adjoint run
 #define REED_MAXNB 12           // Tersoff neighbours per atom held in shared memory
 #define REED_MAXNB_PAIR 64      // pair-potential neighbours per atom held in shared memory
 #define REED_FAST_NB 4          // Tersoff atoms with at most this many list neighbours take the unrolled path

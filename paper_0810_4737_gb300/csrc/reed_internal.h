@@ -19,7 +19,7 @@ size_t track_smem_bytes(int tt, int na, int bond_cap, int adj, int nbins, int ac
 size_t spill_bytes(int tt);
 size_t adj_scratch_bytes(const DevParams& P, size_t entry);
 size_t entry_bytes(int tt, int na);
-cudaError_t occupancy(int tt, int threads, size_t smem, int* ctas, int adj = 0);
+cudaError_t occupancy(int tt, int threads, size_t smem, int* ctas, int adj, int act_cap);
 cudaError_t launch_track(int tt, const DevParams& P, const DevBuf& B, const LaunchCfg& L, cudaStream_t s);
 cudaError_t launch_forces(int tt, const DevParams& P, int n, const double* xyz, const int* sp, const double* ion,
                           double* out, unsigned char* spill, size_t smem, cudaStream_t s);
@@ -35,7 +35,7 @@ size_t track_smem_bytes(int tt, int na, int bond_cap, int adj, int nbins, int ac
 size_t spill_bytes(int tt);
 size_t adj_scratch_bytes(const DevParams& P, size_t entry);
 size_t entry_bytes(int tt, int na);
-cudaError_t occupancy(int tt, int threads, size_t smem, int* ctas, int adj = 0);
+cudaError_t occupancy(int tt, int threads, size_t smem, int* ctas, int adj, int act_cap);
 cudaError_t launch_track(int tt, const DevParams& P, const DevBuf& B, const LaunchCfg& L, cudaStream_t s);
 cudaError_t launch_forces(int tt, const DevParams& P, int n, const double* xyz, const int* sp, const double* ion,
                           double* out, unsigned char* spill, size_t smem, cudaStream_t s);

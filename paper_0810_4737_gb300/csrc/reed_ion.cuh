@@ -82,14 +82,6 @@ template <typename R> __device__ __forceinline__ R lane_of(const R x[3], int lan
 }
 __device__ __forceinline__ int lane_of(const int x[3], int lane) { return lane == 0 ? x[0] : (lane == 1 ? x[1] : x[2]); }
 
-// x^2 + y^2 + z^2 in fixed roundings: whether an atom lies within the cutoff
-// is the same wherever it is asked, and so are a track's bits.
-template <typename R> __device__ __forceinline__ R dist2(R x, R y, R z) { return fma(z, z, fma(x, x, y * y)); }
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
-
 // Largest of the lanes' values; they are >= 0 and not NaN, so their bit
 // patterns order like the numbers.
 __device__ __forceinline__ float warp_max_pos(float x)
@@ -234,11 +226,6 @@ __device__ __forceinline__ bool regs_prologue(const DevParams& P, const HotParam
     regs_frame<R>(P, I, thr, nthr, lane);
     return true;
 }
-
-// Whether an atom is of species 1, and the parameter of its species (no
-// conversion and no indexed constant load: both stall a lone warp).
-template <typename R> __device__ __forceinline__ bool is_second(const V4<R>& p) { return p.w == R(1) || p.w == R(3); }
-template <typename R> __device__ __forceinline__ R of_species(const R q[2], const V4<R>& p) { return is_second(p) ? q[1] : q[0]; }
 
 // The force on an atom from its pair term.
 template <typename R> __device__ __forceinline__ void pair_term_force(const V4<R>& t, R& fx, R& fy, R& fz)

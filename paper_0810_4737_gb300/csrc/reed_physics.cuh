@@ -7,6 +7,18 @@
 
 #include "reed_common.cuh"
 
+// Products and sums that stay out of a fused multiply-add.  Where a sum of
+// products can be fused in more than one way, the potentials below say which
+// (fma, mul_rn, add_rn), so that a pair's bits -- and with them a whole
+// track's, which amplifies any difference -- are the same in every kernel that
+// evaluates it.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+// x^2 + y^2 + z^2
+template <typename R> __device__ __forceinline__ R dist2(R x, R y, R z) { return fma(z, z, fma(x, x, mul_rn(y, y))); }
+
 // ZBL universal screening (Sec. 2 "First"; Ziegler, Biersack, Littmark 1985):
 // phi(x) = sum_i c_i exp(-d_i x) with x = r / a_U,
 // c = {0.18175, 0.50986, 0.28022, 0.02817}, d = {3.1998, 0.94229, 0.4029, 0.20162}.
@@ -14,17 +26,24 @@
 template <typename R> struct Zbl {
     __device__ static __forceinline__ void eval(R r, R ir, R k, R ia, R& V, R& dV)
     {
+        R kr, phi;
+        eval(r, ir, k, ia, V, dV, kr, phi);
+    }
+    // the same with V's two factors
+    __device__ static __forceinline__ void eval(R r, R ir, R k, R ia, R& V, R& dV, R& kr, R& phi)
+    {
         const R x = r * ia;
         const R e0 = Mth<R>::exp2n(R(-3.19980 * 1.4426950408889634) * x);
         const R e1 = Mth<R>::exp2n(R(-0.94229 * 1.4426950408889634) * x);
         const R e2 = Mth<R>::exp2n(R(-0.40290 * 1.4426950408889634) * x);
         const R e3 = Mth<R>::exp2n(R(-0.20162 * 1.4426950408889634) * x);
-        const R phi = R(0.18175) * e0 + R(0.50986) * e1 + R(0.28022) * e2 + R(0.02817) * e3;
-        const R dphi = -(R(0.18175 * 3.19980) * e0 + R(0.50986 * 0.94229) * e1 +
-                         R(0.28022 * 0.40290) * e2 + R(0.02817 * 0.20162) * e3);
-        const R kr = k * ir;
-        V = kr * phi;
-        dV = kr * (dphi * ia - phi * ir);
+        phi = fma(R(0.02817), e3, fma(R(0.28022), e2, fma(R(0.18175), e0, mul_rn(R(0.50986), e1))));
+        const R dphi = -fma(R(0.02817 * 0.20162), e3,
+                            fma(R(0.28022 * 0.40290), e2,
+                                fma(R(0.18175 * 3.19980), e0, mul_rn(R(0.50986 * 0.94229), e1))));
+        kr = mul_rn(k, ir);
+        V = mul_rn(kr, phi);
+        dV = mul_rn(kr, fma(dphi, ia, -mul_rn(phi, ir)));
     }
 };
 
@@ -125,21 +144,25 @@ template <typename R> __device__ __forceinline__ R ters_b(const HotParams<R>& H,
 
 // V_ab at fixed bond order b, given fc(r) and its derivative: value V,
 // radial derivative dV, and pre_fA = (1 - s) fc fA (the coefficient of b in V_ab).
-template <typename R>
+// FAST: the roundings of the one-thread centres (the ZBL energy enters the
+// blend's derivative unrounded), else those of the lane groups.
+template <typename R, bool FAST>
 __device__ __forceinline__ void ters_pair(const HotParams<R>& H, R r, R fc, R dfc, R b, R& V, R& dV, R& pre_fA)
 {
     const R fR = H.tA * Mth<R>::exp(-H.tl1 * r);
     const R fA = -H.tB * Mth<R>::exp(-H.tl2 * r);
-    const R VT = fc * (fR + b * fA);
+    const R VT = mul_rn(fc, fma(b, fA, fR));
     const R dVT = dfc * (fR + b * fA) - fc * (H.tl1 * fR + b * H.tl2 * fA);
     R ds;
     const R s = taper<R>(r, H.t_blo, H.t_binvw, ds);
     pre_fA = (R(1) - s) * fc * fA;
     if (s > R(0)) {
-        R Vz, dVz;
-        Zbl<R>::eval(r, Mth<R>::rcp(r), H.t_zk, H.t_zia, Vz, dVz);
-        V = (R(1) - s) * VT + s * Vz;
-        dV = (R(1) - s) * dVT + ds * (Vz - VT) + s * dVz;
+        R Vz, dVz, kr, phi;
+        Zbl<R>::eval(r, Mth<R>::rcp(r), H.t_zk, H.t_zia, Vz, dVz, kr, phi);
+        const R os = R(1) - s;
+        V = fma(os, VT, mul_rn(s, Vz));
+        const R diff = FAST ? fma(kr, phi, -VT) : add_rn(Vz, -VT);
+        dV = fma(s, dVz, fma(os, dVT, mul_rn(ds, diff)));
     } else {
         V = VT;
         dV = dVT;
@@ -154,11 +177,15 @@ template <typename R> __device__ __forceinline__ R buck_pair(const HotParams<R>&
     const R ir = Mth<R>::rsqrt(r2);
     const R r = r2 * ir;
     R Vb = R(0), dVb = R(0);
-    if (H.bA[p] != R(0) || H.bC[p] != R(0)) {
-        const R e = H.bA[p] * Mth<R>::exp(-r * H.brho_inv[p]);
-        const R ir2 = ir * ir, ir6 = ir2 * ir2 * ir2;
-        Vb = e - H.bC[p] * ir6;
-        dVb = -e * H.brho_inv[p] + R(6) * H.bC[p] * ir6 * ir;
+    // (selected, not indexed: lanes of a warp hold different species pairs, and
+    // an indexed constant load is replayed for each)
+    const R A = p == 1 ? H.bA[1] : (p == 2 ? H.bA[2] : H.bA[0]), C = p == 1 ? H.bC[1] : (p == 2 ? H.bC[2] : H.bC[0]);
+    const R rho_inv = p == 1 ? H.brho_inv[1] : (p == 2 ? H.brho_inv[2] : H.brho_inv[0]);
+    if (A != R(0) || C != R(0)) {
+        const R e = mul_rn(A, Mth<R>::exp(-r * rho_inv));
+        const R ir2 = mul_rn(ir, ir), ir6 = mul_rn(mul_rn(ir2, ir2), ir2);
+        Vb = fma(-C, ir6, e);
+        dVb = fma(mul_rn(mul_rn(R(6), C), ir6), ir, mul_rn(-e, rho_inv));
     }
     R ds;
     const R s = taper<R>(r, H.b_lo, H.b_binvw, ds);
@@ -166,11 +193,12 @@ template <typename R> __device__ __forceinline__ R buck_pair(const HotParams<R>&
     if (s > R(0)) {
         R Vz, dVz;
         Zbl<R>::eval(r, ir, H.b_zk[p], H.b_zia[p], Vz, dVz);
-        V = (R(1) - s) * Vb + s * Vz;
-        dV = (R(1) - s) * dVb + ds * (Vz - Vb) + s * dVz;
+        const R os = R(1) - s;
+        V = fma(os, Vb, mul_rn(s, Vz));
+        dV = fma(s, dVz, fma(os, dVb, mul_rn(ds, Vz - Vb)));
     }
     R dS;
     const R S = taper<R>(r, H.b_rt, H.b_rinvw, dS);
     U = V * S;
-    return (dV * S + V * dS) * ir;
+    return mul_rn(fma(V, dS, mul_rn(dV, S)), ir);
 }

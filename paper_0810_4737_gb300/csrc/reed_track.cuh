@@ -70,15 +70,15 @@ template <typename R> struct TrackShared {
     long long rec_index;
     R xbi[3], vbi[3], ubi[3], vh[3], irel[3], vub, k1;
     double gth[8];
-    R adj_red[REED_MAX_WARPS][12];
+    R adj_red[REED_ADJ_WARPS][12];
     int Aold[3];
     int shift, event, status, src, top, nclone, slot;
     int need_count, active_count;
     int nhit0;            // ion-target-only model: atoms within the cutoff at the last list build
-    unsigned long long cnt[ION_NCOUNT];   // ion-target-only model: counters of this CTA, flushed at exit
+    unsigned long long cnt[REED_NCOUNT];  // counters of this CTA (C_*; ion-target-only model: ION_*), flushed at exit
+    long long t_mark;     // clock of the last lap
     int nspill;           // overflow rows taken by the current lists
     int ncls[4];          // Tersoff: slots per centre-pass class, in `order` (see ters_centres)
-    unsigned long long cls_sum[4];   // centre evaluations per class, summed over passes (thread 0)
     // Tersoff partial refreshes: atoms whose bins are stale since the last
     // full build (atom order), and the atoms refreshed now
     int nstale, nhot;
@@ -429,6 +429,10 @@ __device__ __forceinline__ void deposit_damage(const DevParams& P, const DevBuf&
 }
 template <typename R> __device__ __forceinline__ bool is_active(const V4<R>& p) { return p.w >= R(0) && p.w < R(2); }
 template <typename R> __device__ __forceinline__ int species_of(const V4<R>& p) { return ((int)p.w) & 1; }
+// Whether an atom is of species 1, and the parameter of its species (no
+// conversion and no indexed constant load: both stall a warp).
+template <typename R> __device__ __forceinline__ bool is_second(const V4<R>& p) { return p.w == R(1) || p.w == R(3); }
+template <typename R> __device__ __forceinline__ R of_species(const R q[2], const V4<R>& p) { return is_second(p) ? q[1] : q[0]; }
 
 // ---------------------------------------------------------------------------
 // ---------------------------------------------------------------------------
@@ -855,7 +859,7 @@ __device__ void finish_tersoff_lists(const DevParams& P, Win<R, TT>& W, int nact
 
 template <typename R, int TT>
 __device__ void build_neighbours(const DevParams& P, const HotParams<R>& H, Win<R, TT>& W, int& overflow,
-                                 int& cap_overflow, unsigned long long& spilled)
+                                 int& cap_overflow)
 {
     const int na = P.na, nbins = P.g_nbins;
     TrackShared<R>* S = W.S;
@@ -936,7 +940,7 @@ __device__ void build_neighbours(const DevParams& P, const HotParams<R>& H, Win<
         // pair potentials need lists of the integrated atoms only
         if (threadIdx.x == 0) {
             S->need_count = nact_slots;
-            spilled += (unsigned long long)min(S->nspill, REED_SPILL_ROWS);
+            S->cnt[C_SPILLED] += (unsigned long long)min(S->nspill, REED_SPILL_ROWS);
         }
         __syncthreads();
         return;
@@ -967,7 +971,7 @@ __device__ void build_neighbours(const DevParams& P, const HotParams<R>& H, Win<
     __syncthreads();
     if (threadIdx.x == 0) {
         S->need_count = nneed;
-        spilled += (unsigned long long)min(S->nspill, REED_SPILL_ROWS);
+        S->cnt[C_SPILLED] += (unsigned long long)min(S->nspill, REED_SPILL_ROWS);
     }
     finish_tersoff_lists<R, TT>(P, W, nact_slots, nneed, overflow);
 }
@@ -991,8 +995,7 @@ __device__ void build_neighbours(const DevParams& P, const HotParams<R>& H, Win<
 // overflow; the caller then builds from scratch.
 // ---------------------------------------------------------------------------
 template <typename R, int TT>
-__device__ bool refresh_lists(const DevParams& P, const HotParams<R>& H, Win<R, TT>& W, int& overflow,
-                              unsigned long long& spilled)
+__device__ bool refresh_lists(const DevParams& P, const HotParams<R>& H, Win<R, TT>& W, int& overflow)
 {
     const int na = P.na, tid = threadIdx.x, lane = tid & 31, nw = blockDim.x >> 5, wid = tid >> 5;
     TrackShared<R>* S = W.S;
@@ -1134,7 +1137,7 @@ __device__ bool refresh_lists(const DevParams& P, const HotParams<R>& H, Win<R, 
     __syncthreads();
     if (tid == 0) {
         S->need_count = nneed;
-        spilled += (unsigned long long)(min(S->nspill, REED_SPILL_ROWS) - min(nsp0, REED_SPILL_ROWS));
+        S->cnt[C_SPILLED] += (unsigned long long)(min(S->nspill, REED_SPILL_ROWS) - min(nsp0, REED_SPILL_ROWS));
     }
     // (pending marks set by the new rows' lists are not needed: clear them)
     for (int i = i0; i < i1; ++i)
@@ -1170,7 +1173,7 @@ __device__ bool refresh_lists(const DevParams& P, const HotParams<R>& H, Win<R, 
 // listed, and no listed pair may be farther than r_list + skin.  Counts the
 // differences.
 template <typename R, int TT>
-__device__ void check_lists(const DevParams& P, const HotParams<R>& H, Win<R, TT>& W, R r2ok, unsigned long long& errors)
+__device__ __noinline__ void check_lists(const DevParams& P, const HotParams<R>& H, Win<R, TT> W, R r2ok)
 {
     if constexpr (TT != REED_TT_TERSOFF) return;   // (the pair lists are neighbour-major)
     const R rmax = Mth<R>::rsqrt(H.rlist2);
@@ -1190,7 +1193,7 @@ __device__ void check_lists(const DevParams& P, const HotParams<R>& H, Win<R, TT
         }
         for (int q = 0; q < m; ++q) e += list_d2(pa, W.pos[row[q]]) < lim ? 0 : 1;
     }
-    errors += e;
+    if (e) atomicAdd(&W.S->cnt[C_NLCHECK], e);
     __syncthreads();
 }
 
@@ -1216,7 +1219,7 @@ __device__ void check_lists(const DevParams& P, const HotParams<R>& H, Win<R, TT
 // (unrolled; missing neighbours have fc = P = Q = 0 and contribute nothing).
 template <typename R, int TT>
 __device__ __forceinline__ R ters_centre_fast(const HotParams<R>& H, Win<R, TT>& W, int k, int m, int nact,
-                                              unsigned long long& triplets)
+                                              unsigned& triplets)
 {
     constexpr int M = REED_FAST_NB;
     const int a = W.slot_atom[k];
@@ -1244,7 +1247,7 @@ __device__ __forceinline__ R ters_centre_fast(const HotParams<R>& H, Win<R, TT>&
             npos += (fc[q] > R(0) || dfc[q] != R(0)) ? 1 : 0;
         }
     }
-    if (m > 1) triplets += (unsigned long long)((m - 1) * npos);
+    if (m > 1) triplets += (unsigned)((m - 1) * npos);
     // angle terms of every pair of neighbours
     R c[M][M], g[M][M], dg[M][M];
 #pragma unroll
@@ -1267,7 +1270,7 @@ __device__ __forceinline__ R ters_centre_fast(const HotParams<R>& H, Win<R, TT>&
         if (q < m && (fc[q] > R(0) || dfc[q] != R(0))) {
             R db, V, dV, pfa;
             const R b = ters_b<R>(H, zeta, db);
-            ters_pair<R>(H, rr[q], fc[q], dfc[q], b, V, dV, pfa);
+            ters_pair<R, true>(H, rr[q], fc[q], dfc[q], b, V, dV, pfa);
             P[q] = R(0.5) * pfa * db;
             Q[q] = R(0.5) * dV;
             E += R(0.5) * V;
@@ -1328,7 +1331,7 @@ __device__ __forceinline__ R ters_centre_fast(const HotParams<R>& H, Win<R, TT>&
 // group; sums over the group use the fixed butterfly order.  All 32 lanes of
 // the warp call it together, each group with its own slot k (k < 0: idle).
 template <typename R, int TT, int G>
-__device__ R ters_centre_group(const HotParams<R>& H, Win<R, TT>& W, int k, int nact, unsigned long long& triplets)
+__device__ R ters_centre_group(const HotParams<R>& H, Win<R, TT>& W, int k, int nact, unsigned& triplets)
 {
     constexpr int NH = G == 32 ? 2 : 1;
     constexpr unsigned FULL = 0xffffffffu;
@@ -1372,7 +1375,7 @@ __device__ R ters_centre_group(const HotParams<R>& H, Win<R, TT>& W, int k, int 
         }
         npos += __popc(__ballot_sync(FULL, ok[h] && (fc[h] > R(0) || dfc[h] != R(0))) & gmask);
     }
-    if (lg == 0 && m > 1) triplets += (unsigned long long)((m - 1) * npos);
+    if (lg == 0 && m > 1) triplets += (unsigned)((m - 1) * npos);
     // bond orders of this lane's bonds
     R zeta[NH];
 #pragma unroll
@@ -1396,7 +1399,7 @@ __device__ R ters_centre_group(const HotParams<R>& H, Win<R, TT>& W, int k, int 
         if (ok[h] && (fc[h] > R(0) || dfc[h] != R(0))) {
             R db, V, dV, pfa;
             const R b = ters_b<R>(H, zeta[h], db);
-            ters_pair<R>(H, rr[h], fc[h], dfc[h], b, V, dV, pfa);
+            ters_pair<R, false>(H, rr[h], fc[h], dfc[h], b, V, dV, pfa);
             P[h] = R(0.5) * pfa * db;
             Q[h] = R(0.5) * dV;
             E += R(0.5) * V;
@@ -1468,7 +1471,7 @@ __device__ R ters_centre_group(const HotParams<R>& H, Win<R, TT>& W, int k, int 
 // warps from the last one down (the last warps have the fewest one-thread
 // slots).  Returns this thread's share of the Tersoff energy.
 template <typename R, int TT>
-__device__ R ters_centres(const HotParams<R>& H, Win<R, TT>& W, unsigned long long& triplets)
+__device__ R ters_centres(const HotParams<R>& H, Win<R, TT>& W, unsigned& triplets)
 {
     const int nact = W.S->active_count;
     const int n0 = W.S->ncls[0], n1 = W.S->ncls[1], n2 = W.S->ncls[2], n3 = W.S->ncls[3];
@@ -1520,27 +1523,36 @@ __device__ __forceinline__ void ters_gather(const Win<R, TT>& W, int k, R& Fx, R
 }
 
 // Buckingham / short-range pair forces on atom i from its list (each pair is
-// visited from both ends; the energy is halved).
-template <typename R, int TT>
-__device__ R pair_force(const HotParams<R>& H, Win<R, TT>& W, int i, int k, R& Fx, R& Fy, R& Fz)
+// visited from both ends; the energy is halved).  The atoms of four entries
+// are loaded at a time, so that their loads overlap; the forces are added in
+// list order.
+template <typename R, int TT, bool ENERGY>
+__device__ __forceinline__ R pair_force(const HotParams<R>& H, Win<R, TT>& W, int i, int k, R& Fx, R& Fy, R& Fz)
 {
     const int m = W.nnb[k];
     const V4<R> pi = W.pos[i];
-    const int si = species_of(pi);
+    const int si = is_second(pi);
     const uint16_t* nb = W.list(k, m);
     const int oq = m <= maxnb(TT) ? W.nb_q : 1;   // an overflow row is contiguous
     R E = R(0);
-    for (int q = 0; q < m; ++q) {
-        const V4<R> pj = W.pos[nb[(size_t)q * oq]];
-        R dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
-        R r2 = dx * dx + dy * dy + dz * dz;
-        if (r2 >= H.b_rc2) continue;
-        R U;
-        R g = buck_pair<R>(H, si + species_of(pj), r2, U);
-        Fx += g * dx;
-        Fy += g * dy;
-        Fz += g * dz;
-        E += R(0.5) * U;
+    for (int q0 = 0; q0 < m; q0 += 4) {
+        V4<R> pp[4];
+        const int left = m - q0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) pp[u] = W.pos[u < left ? (int)nb[(size_t)(q0 + u) * oq] : i];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const V4<R> pj = pp[u];
+            const R dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
+            const R r2 = dist2(dx, dy, dz);
+            if (u >= left || r2 >= H.b_rc2) continue;
+            R U;
+            const R g = buck_pair<R>(H, si + is_second(pj), r2, U);
+            Fx += g * dx;
+            Fy += g * dy;
+            Fz += g * dz;
+            if (ENERGY) E += R(0.5) * U;
+        }
     }
     return E;
 }
@@ -1550,15 +1562,6 @@ template <typename R> struct Partial {
     R fx, fy, fz, rho, vmax2, epot;
     int pairs, bonds;
     R pmax;
-};
-
-// Per-thread work counters (algorithmic units of a step, see stats).
-struct WorkCount {
-    unsigned long long triplets = 0;   // Tersoff bond-angle terms (one per zeta term)
-    unsigned long long moved = 0;      // integrated atom updates
-    unsigned long long spilled = 0;    // overflow rows taken by list builds (thread 0)
-    unsigned long long refreshes = 0;  // Tersoff partial refreshes (thread 0)
-    unsigned long long nl_errors = 0;  // list self-check differences (all threads)
 };
 
 // Force evaluation over the whole window; with KICK the second half kick is
@@ -1573,7 +1576,7 @@ __device__ __forceinline__ void atom_force(const DevParams& P, const HotParams<R
     const R ix = W.S->rel[0], iy = W.S->rel[1], iz = W.S->rel[2];
     V4<R> p = W.pos[i];
     const bool act = is_active(p);
-    R fx = R(0), fy = R(0), fz = R(0);
+    R fx = R(0), fy = R(0), fz = R(0), term = R(0);
     if (TT == REED_TT_TERSOFF && act && k >= 0) {   // the bonds centred on i, from the centre pass
         const V4<R> f1 = W.frc[i];
         fx = f1.x;
@@ -1584,7 +1587,8 @@ __device__ __forceinline__ void atom_force(const DevParams& P, const HotParams<R
     const R r2 = dx * dx + dy * dy + dz * dz;
     if (r2 < H.rc2) {
         R U, rw;
-        const R g = ion_pair<R>(H, P.spline_on, P.rho_on, species_of(p), r2, U, rw);
+        const R g = ion_pair<R>(H, P.spline_on, P.rho_on, is_second(p), r2, U, rw);
+        term = g;
         fx -= g * dx;
         fy -= g * dy;
         fz -= g * dz;
@@ -1604,7 +1608,8 @@ __device__ __forceinline__ void atom_force(const DevParams& P, const HotParams<R
         }
         if constexpr (TT == REED_TT_BUCKINGHAM) {
             if (act || want_energy) {
-                out.epot += pair_force<R, TT>(H, W, i, k, fx, fy, fz);
+                const R e = pair_force<R, TT, !KICK>(H, W, i, k, fx, fy, fz);
+                if (!KICK) out.epot += e;
                 out.bonds += W.nnb[k];
             }
         }
@@ -1613,11 +1618,11 @@ __device__ __forceinline__ void atom_force(const DevParams& P, const HotParams<R
     f.x = fx;
     f.y = fy;
     f.z = fz;
-    f.w = R(0);
+    f.w = term;   // the pair term with the ion, for sum_ion_terms
     W.frc[i] = f;
     if (KICK && act) {
         V4<R> v = W.vel[i];
-        const R kk = hdt * H.invM2[species_of(p)];
+        const R kk = hdt * of_species(H.invM2, p);
         v.x += kk * fx;
         v.y += kk * fy;
         v.z += kk * fz;
@@ -1647,9 +1652,11 @@ __device__ void force_phase(const DevParams& P, const HotParams<R>& H, Win<R, TT
                 // matters (its own force is never used)
                 const R dx = p.x - W.S->rel[0], dy = p.y - W.S->rel[1], dz = p.z - W.S->rel[2];
                 const R r2 = dx * dx + dy * dy + dz * dz;
+                W.frc[i].w = R(0);
                 if (r2 < H.rc2) {
                     R U, rw;
-                    const R g = ion_pair<R>(H, P.spline_on, P.rho_on, species_of(p), r2, U, rw);
+                    const R g = ion_pair<R>(H, P.spline_on, P.rho_on, is_second(p), r2, U, rw);
+                    W.frc[i].w = g;
                     out.fx += g * dx;
                     out.fy += g * dy;
                     out.fz += g * dz;
@@ -1663,6 +1670,58 @@ __device__ void force_phase(const DevParams& P, const HotParams<R>& H, Win<R, TT
             if (is_active(p) && sl < (unsigned)nact) continue;   // done above
             const int k = (sl < REED_PENDING && want_energy) ? (int)sl : -1;
             atom_force<R, TT, KICK>(P, H, W, i, k, hdt, out, want_energy);
+        }
+    }
+}
+
+// Partial sums of the force on the ion and of the local density, taken over
+// the atoms by vt virtual threads when the CTA has another number of threads:
+// the pair terms wait in frc.w, virtual thread t adds those of list slots t, t
+// + vt, ... and then of the other atoms t, t + vt, ..., and 32 consecutive
+// virtual threads are one row of S->red -- the summation order of a CTA of vt
+// threads (threads_per_track).  All threads, after a barrier; a barrier must
+// follow.  (vmax2, pmax and the counts of the CTA's own warps are in the same
+// rows: their order does not matter.)
+template <typename R>
+__device__ __noinline__ void sum_ion_terms(const DevParams& P, TrackShared<R>* S, const V4<R>* pos, const V4<R>* frc,
+                                           const uint16_t* slot_atom, const uint16_t* need_map, int vt)
+{
+    const HotParams<R>& H = hot<R>(P);
+    const int lane = threadIdx.x & 31, nact = S->active_count;
+    const R ix = S->rel[0], iy = S->rel[1], iz = S->rel[2];
+    for (int vw = threadIdx.x >> 5; vw < (vt >> 5); vw += blockDim.x >> 5) {
+        R fx = R(0), fy = R(0), fz = R(0), rho = R(0);
+        auto add = [&](int i) {
+            const V4<R> p = pos[i];
+            const R g = frc[i].w, dx = p.x - ix, dy = p.y - iy, dz = p.z - iz;
+            fx += g * dx;
+            fy += g * dy;
+            fz += g * dz;
+            if (P.rho_on) {
+                const R r2 = dx * dx + dy * dy + dz * dz;
+                R U, rw;
+                if (r2 < H.rc2) {
+                    ion_pair<R>(H, P.spline_on, P.rho_on, is_second(p), r2, U, rw);
+                    rho += rw;
+                }
+            }
+        };
+        for (int k = vw * 32 + lane; k < nact; k += vt) add(slot_atom[k]);
+        if (P.margin)
+            for (int i = vw * 32 + lane; i < P.na; i += vt) {
+                const V4<R> p = pos[i];
+                if (is_present(p) && !(is_active(p) && (unsigned)need_map[i] < (unsigned)nact)) add(i);
+            }
+        fx = warp_sum(fx);
+        fy = warp_sum(fy);
+        fz = warp_sum(fz);
+        rho = warp_sum(rho);
+        if (lane == 0) {
+            R* row = S->red[vw];
+            row[0] = fx;
+            row[1] = fy;
+            row[2] = fz;
+            row[3] = rho;
         }
     }
 }
@@ -1683,16 +1742,18 @@ __device__ __forceinline__ void reduce_partials(Win<R, TT>& W, Partial<R>& q)
 }
 
 // Sum the per-warp partials (thread 0), fixed order; rows 4 and 8 are maxima.
+// nv: rows of the ion's sums (0-3); the others have one row per warp.
 template <typename R, int TT>
-__device__ __forceinline__ void gather_partials(Win<R, TT>& W, R out[REED_NRED])
+__device__ __forceinline__ void gather_partials(Win<R, TT>& W, R out[REED_NRED], int nv)
 {
     const int nw = (blockDim.x + 31) >> 5;
     R acc[REED_NRED];
 #pragma unroll
     for (int c = 0; c < REED_NRED; ++c) acc[c] = R(0);
-    for (int w = 0; w < nw; ++w) {
+    for (int w = 0; w < max(nw, nv); ++w) {
         const R* row = W.S->red[w];
         for (int c = 0; c < REED_NRED; ++c) {
+            if (w >= (c < 4 ? nv : nw)) continue;
             if (c == 4 || c == 8) acc[c] = max(acc[c], row[c]);
             else acc[c] += row[c];
         }
@@ -1997,30 +2058,34 @@ __device__ __forceinline__ void copy_window(const DevParams& P, Win<R, TT>& W, u
 
 // Forces + (optionally) target bookkeeping at the start of a track.
 template <typename R, int TT>
-__device__ void initial_forces(const DevParams& P, const HotParams<R>& H, Win<R, TT>& W, unsigned long long& ctr_bonds,
-                               unsigned long long& ctr_rebuild, int& nbovf, int& capovf, WorkCount& wc)
+__device__ void initial_forces(const DevParams& P, const HotParams<R>& H, Win<R, TT>& W, int& nbovf, int& capovf,
+                               unsigned& triplets, int vt)
 {
-    build_neighbours<R, TT>(P, H, W, nbovf, capovf, wc.spilled);
-    if (threadIdx.x == 0) ++ctr_rebuild;
+    build_neighbours<R, TT>(P, H, W, nbovf, capovf);
+    if (threadIdx.x == 0) ++W.S->cnt[C_REBUILDS];
     __syncthreads();
-    if (P.nl_check) check_lists<R, TT>(P, H, W, H.rlist2, wc.nl_errors);
+    if (P.nl_check) check_lists<R, TT>(P, H, W, H.rlist2);
     if constexpr (TT == REED_TT_TERSOFF) {
-        ters_centres<R, TT>(H, W, wc.triplets);
+        ters_centres<R, TT>(H, W, triplets);
         __syncthreads();
     }
     Partial<R> q = {R(0), R(0), R(0), R(0), R(0), R(0), 0, 0};
     force_phase<R, TT, false>(P, H, W, R(0), q, false);
     reduce_partials<R, TT>(W, q);
     __syncthreads();
+    if (vt != (int)blockDim.x) {
+        sum_ion_terms<R>(P, W.S, W.pos, W.frc, W.slot_atom, W.need_map, vt);
+        __syncthreads();
+    }
     if (threadIdx.x == 0) {
         R red[REED_NRED];
-        gather_partials<R, TT>(W, red);
+        gather_partials<R, TT>(W, red, vt >> 5);
         IonState<R>& I = W.S->ion;
         I.f[0] = red[0];
         I.f[1] = red[1];
         I.f[2] = red[2];
         I.rho = red[3];
-        ctr_bonds += (unsigned long long)red[7];
+        W.S->cnt[C_BONDS] += (unsigned long long)red[7];
     }
     __syncthreads();
 }
@@ -2035,13 +2100,25 @@ __device__ void initial_forces(const DevParams& P, const HotParams<R>& H, Win<R,
 // ---------------------------------------------------------------------------
 template <typename R, int TT> constexpr int track_min_ctas() { return TT == REED_TT_TERSOFF && sizeof(R) == 4 ? 2 : 1; }
 
-// Threads per track at most: 512 for the pair-list model (one track fills an
-// SM's shared memory, so its warps are all the SM gets), else 256.
-template <int TT> constexpr int track_max_threads() { return TT == REED_TT_BUCKINGHAM ? 512 : 256; }
+// Threads of a track's CTA at most.  The pair-list model: one track fills an
+// SM's shared memory, so its warps are all that the SM gets -- 24 of them, one
+// thread per atom of a 4^3-cell CeO2 window, in the mixed form (the pair loop
+// needs under 85 registers); the FP64 form is bound by its pipe and keeps 16.
+template <typename R, int TT> constexpr int track_max_threads()
+{
+    return TT == REED_TT_BUCKINGHAM ? (sizeof(R) == 4 ? 768 : 512) : 256;
+}
+// Threads of a CTA whose run sums by vt virtual threads.
+template <typename R, int TT> inline int track_threads(int act_cap)
+{
+    if (TT == REED_TT_TERSOFF) return 256;
+    const int t = (act_cap + 31) / 32 * 32;
+    return t < 256 ? 256 : (t > track_max_threads<R, TT>() ? track_max_threads<R, TT>() : t);
+}
 
 template <typename R, int TT>
-__global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, TT>())) reed_track_kernel(
-    const __grid_constant__ DevParams P, const __grid_constant__ DevBuf B)
+__global__ void __launch_bounds__((track_max_threads<R, TT>()), (track_min_ctas<R, TT>())) reed_track_kernel(
+    const __grid_constant__ DevParams P, const __grid_constant__ DevBuf B, const int vt)
 {
     static_assert(TT != REED_TT_NONE, "the ion-target-only model has its own kernel");
     extern __shared__ __align__(16) unsigned char smem[];
@@ -2052,24 +2129,20 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
     const int tid = threadIdx.x;
     unsigned char* stack = B.stacks ? B.stacks + (size_t)blockIdx.x * B.stack_stride : nullptr;
 
-    // thread-0 counters, flushed at exit
-    unsigned long long c_prim = 0, c_clone = 0, c_tracks = 0, c_steps = 0, c_pairs = 0, c_bonds = 0,
-                       c_shift = 0, c_rebuild = 0, c_drop = 0, c_fail = 0;
     int nbovf = 0, capovf = 0;
-    WorkCount wc;
+    unsigned triplets = 0;   // bond-angle terms of this thread in the current track
     // phase clocks (thread 0): time between consecutive barriers of a step
-    unsigned long long ph[REED_NPHASE] = {0, 0, 0, 0, 0, 0};
-    long long t_mark = clock64();
     auto lap = [&](int phase) {
         if (tid == 0) {
             const long long now = clock64();
-            ph[phase] += (unsigned long long)(now - t_mark);
-            t_mark = now;
+            S->cnt[C_PHASE0 + phase] += (unsigned long long)(now - S->t_mark);
+            S->t_mark = now;
         }
     };
     if (tid == 0) {
         S->top = 0;
-        for (int c = 0; c < 4; ++c) S->cls_sum[c] = 0;
+        S->t_mark = clock64();
+        for (int c = 0; c < REED_NCOUNT; ++c) S->cnt[c] = 0;
     }
     W.clear_grid(P);
 
@@ -2123,7 +2196,7 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
             if (tid == 0) {
                 launch_primary<R>(P, S->ion, S->pidx);
                 set_frame<R>(P, S);
-                ++c_prim;
+                ++S->cnt[C_PRIMARIES];
             }
             __syncthreads();
             const uint64_t key = S->ion.key;
@@ -2137,7 +2210,7 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
                 W.frc[i] = f;
             }
             __syncthreads();
-            initial_forces<R, TT>(P, H, W, c_bonds, c_rebuild, nbovf, capovf, wc);
+            initial_forces<R, TT>(P, H, W, nbovf, capovf, triplets, vt);
         } else if (src == SRC_STOLEN) {
             const unsigned char* rec = B.pool + (size_t)S->slot * B.entry_bytes;
             if (tid == 0) {
@@ -2155,8 +2228,8 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
                 atomicSub(&B.pool_ctl[1], 1u);
                 if (B.splits) atomicAdd(&B.splits[REED_MAX_THR], 1ull);
             }
-            build_neighbours<R, TT>(P, H, W, nbovf, capovf, wc.spilled);
-            if (tid == 0) ++c_rebuild;
+            build_neighbours<R, TT>(P, H, W, nbovf, capovf);
+            if (tid == 0) ++S->cnt[C_REBUILDS];
             __syncthreads();
         } else {
             unsigned char* rec = stack + (size_t)(S->top - 1) * B.entry_bytes;
@@ -2167,8 +2240,8 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
             copy_window<R, TT>(P, W, rec, false);
             __syncthreads();
             if (tid == 0) S->top -= 1;
-            build_neighbours<R, TT>(P, H, W, nbovf, capovf, wc.spilled);
-            if (tid == 0) ++c_rebuild;
+            build_neighbours<R, TT>(P, H, W, nbovf, capovf);
+            if (tid == 0) ++S->cnt[C_REBUILDS];
             __syncthreads();
         }
         const bool tracing = (src == SRC_PRIMARY) && (S->pidx < P.trace_tracks);
@@ -2193,13 +2266,13 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
             // first kicked at the end of this step, one leaving it still
             // moves in this step)
             R pm1 = R(0), pm2 = R(0);   // this thread's two longest paths
+            if (tid == 0) S->cnt[C_MOVED] += (unsigned)S->active_count;
             for (int i = tid; i < P.na; i += blockDim.x) {
                 V4<R> p = W.pos[i];
                 const bool act = is_active(p);
                 if (!act && !shift) continue;   // frozen atoms do not move
                 V4<R> v = W.vel[i], f = W.frc[i];
                 if (act) {
-                    ++wc.moved;
                     const R k = hdt * H.invM2[species_of(p)];
                     v.x += k * f.x;
                     v.y += k * f.y;
@@ -2248,33 +2321,37 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
             if (shift || m1 + m2 > H.skin) {
                 bool refreshed = false;
                 if constexpr (TT == REED_TT_TERSOFF) {
-                    if (!shift) refreshed = refresh_lists<R, TT>(P, H, W, nbovf, wc.spilled);
+                    if (!shift) refreshed = refresh_lists<R, TT>(P, H, W, nbovf);
                 }
-                if (!refreshed) build_neighbours<R, TT>(P, H, W, nbovf, capovf, wc.spilled);
+                if (!refreshed) build_neighbours<R, TT>(P, H, W, nbovf, capovf);
                 __syncthreads();
-                if (tid == 0) ++(refreshed ? wc.refreshes : c_rebuild);
+                if (tid == 0) ++S->cnt[refreshed ? C_REFRESH : C_REBUILDS];
                 if (P.nl_check)
-                    check_lists<R, TT>(P, H, W, refreshed ? H.tcut * H.tcut : H.rlist2, wc.nl_errors);
+                    check_lists<R, TT>(P, H, W, refreshed ? H.tcut * H.tcut : H.rlist2);
                 lap(PH_BUILD);
             }
             if constexpr (TT == REED_TT_TERSOFF) {
-                ters_centres<R, TT>(H, W, wc.triplets);
+                ters_centres<R, TT>(H, W, triplets);
                 __syncthreads();
                 lap(PH_PASS1);
                 if (tid == 0)
-                    for (int c = 0; c < 4; ++c) S->cls_sum[c] += (unsigned)S->ncls[c];
+                    for (int c = 0; c < 4; ++c) S->cnt[C_CLS0 + c] += (unsigned)S->ncls[c];
             }
             force_phase<R, TT, true>(P, H, W, hdt, q, false);
             reduce_partials<R, TT>(W, q);
             __syncthreads();
+            if (vt != (int)blockDim.x) {
+                sum_ion_terms<R>(P, W.S, W.pos, W.frc, W.slot_atom, W.need_map, vt);
+                __syncthreads();
+            }
             lap(PH_FORCE);
             if (tid == 0) {
                 R red[REED_NRED];
-                gather_partials<R, TT>(W, red);
-                c_pairs += (unsigned long long)red[6];
-                c_bonds += (unsigned long long)red[7];
-                c_shift += shift;
-                ++c_steps;
+                gather_partials<R, TT>(W, red, vt >> 5);
+                S->cnt[C_PAIRS] += (unsigned long long)red[6];
+                S->cnt[C_BONDS] += (unsigned long long)red[7];
+                S->cnt[C_SHIFTS] += (unsigned)shift;
+                ++S->cnt[C_STEPS];
                 int ev = ion_epilogue<R>(P, H, S, red);
                 if (tracing && S->ion.steps <= P.trace_steps) {
                     const IonState<R>& I = S->ion;
@@ -2320,7 +2397,7 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
                         C.id = clone_id(I.id, I.level);
                         C.key = track_key(P.seed, C.id);
                         *reinterpret_cast<IonState<R>*>(rec) = C;
-                        ++c_clone;
+                        ++S->cnt[C_CLONES];
                         if (B.splits) atomicAdd(&B.splits[min(I.level, REED_MAX_THR) - 1], 1ull);
                     }
                     copy_window<R, TT>(P, W, rec, true);
@@ -2335,7 +2412,7 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
                 }
                 if (S->top >= B.stack_depth || stack == nullptr) {
                     if (tid == 0) {
-                        c_drop += (unsigned long long)(nc - c);
+                        S->cnt[C_DROPPED] += (unsigned long long)(nc - c);
                         atomicOr(B.status, ERR_QUEUE);
                         // the track still passes the levels (its depths stay in step with its
                         // weight 2^-level), so the dropped clones' weight is lost from the
@@ -2353,7 +2430,7 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
                     C.id = clone_id(I.id, I.level);
                     C.key = track_key(P.seed, C.id);
                     *reinterpret_cast<IonState<R>*>(rec) = C;
-                    ++c_clone;
+                    ++S->cnt[C_CLONES];
                     if (B.splits) atomicAdd(&B.splits[min(I.level, REED_MAX_THR) - 1], 1ull);
                 }
                 copy_window<R, TT>(P, W, rec, true);
@@ -2377,11 +2454,16 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
         }
         if (tid == 0) {
             if (S->status == REED_TRACK_FAILED) {
-                ++c_fail;
+                ++S->cnt[C_FAILED];
                 atomicOr(B.status, ERR_NONFINITE);
             }
             finish_track<R>(P, B, S->ion, S->status);
-            ++c_tracks;
+            ++S->cnt[C_TRACKS];
+        }
+        if constexpr (TT == REED_TT_TERSOFF) {
+            const unsigned tr = __reduce_add_sync(0xffffffffu, triplets);
+            if ((tid & 31) == 0 && tr) atomicAdd(&S->cnt[C_TRIPLETS], (unsigned long long)tr);
+            triplets = 0;
         }
         __syncthreads();
     }
@@ -2394,33 +2476,9 @@ __global__ void __launch_bounds__((track_max_threads<TT>()), (track_min_ctas<R, 
     }
     if ((tid & 31) == 0 && ov) atomicAdd(&B.counters[C_NBOVF], (unsigned long long)ov);
     if ((tid & 31) == 0 && oc) atomicAdd(&B.counters[C_CAPOVF], (unsigned long long)oc);
-    unsigned long long tr = wc.triplets, mv = wc.moved;
-    for (int o = 16; o > 0; o >>= 1) {
-        tr += __shfl_xor_sync(0xffffffffu, tr, o);
-        mv += __shfl_xor_sync(0xffffffffu, mv, o);
-    }
-    if ((tid & 31) == 0) {
-        if (tr) atomicAdd(&B.counters[C_TRIPLETS], tr);
-        atomicAdd(&B.counters[C_MOVED], mv);
-    }
-    if (tid == 0 && wc.spilled) atomicAdd(&B.counters[C_SPILLED], wc.spilled);
-    if (tid == 0 && wc.refreshes) atomicAdd(&B.counters[C_REFRESH], wc.refreshes);
-    if (TT == REED_TT_TERSOFF && tid == 0)
-        for (int c = 0; c < 4; ++c)
-            if (S->cls_sum[c]) atomicAdd(&B.counters[C_CLS0 + c], S->cls_sum[c]);
-    if (wc.nl_errors) atomicAdd(&B.counters[C_NLCHECK], wc.nl_errors);
-    if (tid == 0) {
-        atomicAdd(&B.counters[C_PRIMARIES], c_prim);
-        atomicAdd(&B.counters[C_CLONES], c_clone);
-        atomicAdd(&B.counters[C_TRACKS], c_tracks);
-        atomicAdd(&B.counters[C_STEPS], c_steps);
-        atomicAdd(&B.counters[C_PAIRS], c_pairs);
-        atomicAdd(&B.counters[C_BONDS], c_bonds);
-        atomicAdd(&B.counters[C_SHIFTS], c_shift);
-        atomicAdd(&B.counters[C_REBUILDS], c_rebuild);
-        atomicAdd(&B.counters[C_DROPPED], c_drop);
-        atomicAdd(&B.counters[C_FAILED], c_fail);
-        lap(PH_ADMIN);
-        for (int k = 0; k < REED_NPHASE; ++k) atomicAdd(&B.counters[C_PHASE0 + k], ph[k]);
-    }
+    __syncthreads();
+    lap(PH_ADMIN);
+    __syncthreads();
+    for (int c = tid; c < REED_NCOUNT; c += blockDim.x)
+        if (S->cnt[c]) atomicAdd(&B.counters[c], S->cnt[c]);
 }
