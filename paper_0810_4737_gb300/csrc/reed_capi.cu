@@ -734,6 +734,7 @@ int reed_run(reed_ctx* ctx, double ion_Z, double ion_M, double energy_eV, double
     if (occ < 1) return fail(ctx, REED_E_SMEM, "kernel does not fit on an SM (%zu B shared, %d threads)", smem, L.threads);
     L.ctas_per_sm = o.ctas_per_sm ? std::min(o.ctas_per_sm, occ) : (tuned ? std::min(ctx->tuned_ctas[pi][ai], occ) : occ);
     L.grid = ctx->sms * L.ctas_per_sm;
+    L.sms = ctx->sms;
 
     // clone stacks: one record per cloning level per CTA
     DevBuf B;
@@ -1623,6 +1624,7 @@ extern "C" int reed_run_static(const reed_lattice* lat, const reed_species* sp, 
                     "than the %zu B static scratch",
                     per_cta * (size_t)desc.sms, desc.sms, P.nthr, B.entry_bytes, B.spill_stride, room);
     L.grid = desc.sms * L.ctas_per_sm;
+    L.sms = desc.sms;
 
     unsigned char* base = nullptr;
     int rc = static_scratch((void**)&base);

@@ -18,6 +18,8 @@
 #define REED_MAX_BASIS 12
 #define REED_MAX_THR 16
 #define REED_MAX_WARPS 24       // warps of a track's CTA at most (768 threads: one per atom of a 4^3-cell CeO2 window)
+#define REED_WIDE 512           // threads of a Tersoff track that has an SM to itself (mixed form)
+#define REED_MAX_TEAM 8         // CTAs that follow one Tersoff track together, at most
 #define REED_ADJ_WARPS 8        // ... of an adjoint run
 #define REED_MAXNB 12           // Tersoff neighbours per atom held in shared memory
 #define REED_MAXNB_PAIR 64      // pair-potential neighbours per atom held in shared memory
@@ -340,9 +342,31 @@ template <typename T> __device__ __forceinline__ T warp_sum(T v)
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-template <typename T> __device__ __forceinline__ T warp_max(T v)
+// The sums of four values over the warp, each added in warp_sum's order: the
+// first two stages halve what a lane carries, so that they take 6 shuffles and
+// not 20.  Lanes 0-7 get the sum of a, 8-15 of b, 16-23 of c, 24-31 of d.
+template <typename T> __device__ __forceinline__ T warp_sum4(T a, T b, T c, T d)
 {
+    constexpr unsigned FULL = 0xffffffffu;
+    const bool h4 = threadIdx.x & 16, h3 = threadIdx.x & 8;
+    const T oa = __shfl_xor_sync(FULL, h4 ? a : c, 16), ob = __shfl_xor_sync(FULL, h4 ? b : d, 16);
+    const T k0 = (h4 ? c : a) + oa, k1 = (h4 ? d : b) + ob;
+    T k = (h3 ? k1 : k0) + __shfl_xor_sync(FULL, h3 ? k0 : k1, 8);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(FULL, k, o);
+    return k;
+}
+// Largest of the lanes' values; they are >= 0 and not NaN, so their bit
+// patterns order like the numbers.
+__device__ __forceinline__ float warp_max_pos(float x)
+{
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x)));
+}
+__device__ __forceinline__ double warp_max_pos(double x)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    return __longlong_as_double((long long)(((unsigned long long)mh << 32) | ml));
 }

@@ -8,7 +8,8 @@
 #include "reed_common.cuh"
 
 struct LaunchCfg {
-    int threads, ctas_per_sm, grid;
+    int threads, ctas_per_sm, grid;   // grid: what buffers are sized for; launch_track may use fewer CTAs
+    int sms;
     size_t smem;
 };
 

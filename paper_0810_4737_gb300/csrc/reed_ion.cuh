@@ -82,21 +82,6 @@ template <typename R> __device__ __forceinline__ R lane_of(const R x[3], int lan
 }
 __device__ __forceinline__ int lane_of(const int x[3], int lane) { return lane == 0 ? x[0] : (lane == 1 ? x[1] : x[2]); }
 
-// Largest of the lanes' values; they are >= 0 and not NaN, so their bit
-// patterns order like the numbers.
-__device__ __forceinline__ float warp_max_pos(float x)
-{
-    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x)));
-}
-__device__ __forceinline__ double warp_max_pos(double x)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
-    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
-    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
-    return __longlong_as_double((long long)(((unsigned long long)mh << 32) | ml));
-}
-
 template <typename R> __device__ __forceinline__ void pack_ion(const IonRegs<R>& I, IonState<R>& s, int lane)
 {
     if (lane < 3) s.x[lane] = I.acc;

@@ -19,12 +19,12 @@
 // paper's result messages, Sec. 3).
 //
 // One step (kick-drift-kick with adaptive dt, Sec. 2):
-//   prologue  (thread 0, FP64) dt from the fastest particle, ion half kick +
-//             drift, window anchor check;
-//   phase A   (all threads) re-anchor moved cells, atom half kick + drift;
+//   prologue  (first warp, a lane per component) dt from the fastest particle,
+//             ion half kick + drift, window anchor check;
+//   phase A   (all threads) atom half kick + drift, re-anchor moved cells;
 //   forces    (all threads) ion-target ZBL, target-target terms, second half
 //             kick of the atoms, per-warp partial sums;
-//   epilogue  (thread 0) ion force reduction, ion second half kick, end /
+//   epilogue  (first warp) ion force reduction, ion second half kick, end /
 //             cloning checks, then straight into the next prologue.
 #pragma once
 
@@ -41,13 +41,13 @@ enum {
     ION_PH_FORCE, ION_PH_ADMIN, ION_NCOUNT
 };
 
-// Ion state as stored in shared memory and in clone records.  Position,
-// time and the energy given to electronic stopping are FP64 accumulators;
-// velocity, force and the step arithmetic are in the force-pass type R, so
-// the mixed form executes only a handful of FP64 additions per step.
+// Ion state as stored in shared memory and in clone records.  Position and
+// time are FP64 accumulators; velocity, force and the step arithmetic are in
+// the force-pass type R, so the mixed form executes only a handful of FP64
+// additions per step.
 template <typename R> struct alignas(16) IonState {
     double x[3];          // absolute position, A
-    double t, e_elec;     // time (tau), energy removed by the drag (eV)
+    double t;             // time (tau)
     R v[3], f[3];         // velocity (A/tau), conservative force (eV/A)
     R vlo[3];             // FP32 form: the rounding error carried with v (v + vlo, see add_velocity)
     R rho, vmax2;         // local density at x; fastest atom's speed^2
@@ -63,6 +63,10 @@ template <typename R> struct TrackShared {
     R dt;
     R rel[3];             // ion position relative to the anchor corner A a
     R zthr, zback, zsurf; // next cloning depth, backscatter plane, surface in the anchor frame
+    int Aold[3];
+    int shift, event, src;
+    long long pidx;
+    // (up to here: what the leader of a team hands to the other CTAs)
     double thr[REED_MAX_THR];  // this track's cloning depths (frozen while it runs)
     int nthr;
     // adjoint workspace
@@ -71,8 +75,10 @@ template <typename R> struct TrackShared {
     R xbi[3], vbi[3], ubi[3], vh[3], irel[3], vub, k1;
     double gth[8];
     R adj_red[REED_ADJ_WARPS][12];
-    int Aold[3];
-    int shift, event, status, src, top, nclone, slot;
+    int near_frozen;      // a frozen atom may come within the cutoff of the ion before the next window move
+    unsigned mark[6];     // clocks: the end of the last step's forces, then of each phase of this step
+    long long moved_from, centred_from, steps_from;   // see count_listed; steps before this CTA took the track
+    int status, top, nclone, slot;
     int need_count, active_count;
     int nhit0;            // ion-target-only model: atoms within the cutoff at the last list build
     unsigned long long cnt[REED_NCOUNT];  // counters of this CTA (C_*; ion-target-only model: ION_*), flushed at exit
@@ -84,8 +90,7 @@ template <typename R> struct TrackShared {
     int nstale, nhot;
     uint16_t stale[REED_MAX_STALE];
     uint16_t hot[REED_MAX_HOT];
-    int scan[4][REED_MAX_WARPS];
-    long long pidx;
+    alignas(16) int scan[REED_MAX_WARPS][4];
     R red[REED_MAX_WARPS][REED_NRED];
     R path2[REED_MAX_WARPS][2];   // per warp: the two longest atom paths since the list build
 };
@@ -151,6 +156,32 @@ template <typename R, int TT> struct Layout {
 #define REED_PENDING 0xFFFEu
 #define REED_NO_REV 0xFFu
 
+// Thread-block clusters.  A barrier of all threads of the cluster, which also
+// orders their shared and global memory accesses.
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ int cluster_rank()
+{
+    int r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ int cluster_size()
+{
+    int r;
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+// p, in the shared memory of this CTA, as an address in that of CTA `rank`
+template <typename T> __device__ __forceinline__ T* in_cta(T* p, int rank)
+{
+    unsigned long long q;
+    asm("mapa.u64 %0, %1, %2;" : "=l"(q) : "l"(p), "r"(rank));
+    return reinterpret_cast<T*>(q);
+}
+
 template <typename R, int TT> struct Win {
     TrackShared<R>* S;
     V4<R>* pos;
@@ -183,6 +214,10 @@ template <typename R, int TT> struct Win {
     // A slot with more neighbours than the shared row holds keeps its whole
     // list in an overflow row; entry 0 of the shared row is then that row's index.
     int nb_slot, nb_q, act_cap;
+    // a track followed by a team of CTAs (see reed_track_kernel): their number,
+    // this one's rank and the distance of their overflow rows
+    int team = 1, rank = 0;
+    long long sp_step = 0;
     // zero the bin counters (all threads; a barrier must follow)
     __device__ void clear_grid(const DevParams& P)
     {
@@ -269,7 +304,38 @@ template <typename R, int TT> struct Win {
     {
         return m <= REED_MAXNB ? rev + (size_t)k * REED_MAXNB : sp_rev + (size_t)nbr[(size_t)k * REED_MAXNB] * REED_SPILL_TERSOFF;
     }
-    // force of the bonds centred on entry e's atom on the integrated atom of slot s
+    // force of the bonds centred on entry e's atom on the integrated atom of slot
+    // s, in the windows of the whole team.  (Its CTAs have the same lists, but an
+    // overflow row's number depends on timing.)
+    template <bool TEAM> __device__ __forceinline__ void put_force(int s, int e, R fx, R fy, R fz) const
+    {
+        if (!TEAM) {
+            bf_store(s, e, fx, fy, fz);
+            return;
+        }
+        const int o = s * REED_BF_STRIDE + e;
+        for (int q = 0; q < team; ++q) {
+            if (nnb[s] <= REED_MAXNB) {
+                *in_cta(bfx + o, q) = fx;
+                *in_cta(bfy + o, q) = fy;
+                *in_cta(bfz + o, q) = fz;
+            } else if (*in_cta(nnb + s, q) > REED_MAXNB) {
+                const int row = *in_cta(nbr + (size_t)s * REED_MAXNB, q);
+                R* b = reinterpret_cast<R*>(reinterpret_cast<unsigned char*>(sp_bf) + (q - rank) * sp_step) +
+                       (size_t)min(row, REED_SPILL_ROWS - 1) * 3 * REED_SPILL_TERSOFF;
+                b[e] = fx;
+                b[REED_SPILL_TERSOFF + e] = fy;
+                b[2 * REED_SPILL_TERSOFF + e] = fz;
+            }
+        }
+    }
+    // force of the bonds centred on the integrated atom a on itself
+    template <bool TEAM> __device__ __forceinline__ void put_centre(int a, const V4<R>& f) const
+    {
+        if (!TEAM) frc[a] = f;
+        else
+            for (int q = 0; q < team; ++q) *in_cta(frc + a, q) = f;
+    }
     __device__ __forceinline__ void bf_store(int s, int e, R fx, R fy, R fz) const
     {
         if (nnb[s] <= REED_MAXNB) {
@@ -710,21 +776,20 @@ __device__ __forceinline__ void block_scan2(TrackShared<R>* S, int c0, int c1, i
         }
     }
     __syncthreads();
-    if (lane == 31) {
-        S->scan[0][wid] = x0;
-        S->scan[1][wid] = x1;
-    }
+    if (lane == 31) *reinterpret_cast<int2*>(S->scan[wid]) = make_int2(x0, x1);
     __syncthreads();
     int b0 = 0, b1 = 0;
     t0 = 0;
     t1 = 0;
+#pragma unroll 4
     for (int w = 0; w < nw; ++w) {
+        const int2 n = *reinterpret_cast<const int2*>(S->scan[w]);
         if (w == wid) {
             b0 = t0;
             b1 = t1;
         }
-        t0 += S->scan[0][w];
-        t1 += S->scan[1][w];
+        t0 += n.x;
+        t1 += n.y;
     }
     o0 = b0 + x0 - c0;
     o1 = b1 + x1 - c1;
@@ -747,20 +812,26 @@ __device__ __forceinline__ void block_scan4(TrackShared<R>* S, const int c[4], i
         }
     }
     __syncthreads();
-    if (lane == 31)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) S->scan[i][wid] = x[i];
+    if (lane == 31) *reinterpret_cast<int4*>(S->scan[wid]) = make_int4(x[0], x[1], x[2], x[3]);
     __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int b = 0, tot = 0;
-        for (int w = 0; w < nw; ++w) {
-            if (w == wid) b = tot;
-            tot += S->scan[i][w];
-        }
-        o[i] = b + x[i] - c[i];
-        t[i] = tot;
+    int4 b = make_int4(0, 0, 0, 0), n = b;
+#pragma unroll 4
+    for (int w = 0; w < nw; ++w) {
+        const int4 q = *reinterpret_cast<const int4*>(S->scan[w]);
+        if (w == wid) b = n;
+        n.x += q.x;
+        n.y += q.y;
+        n.z += q.z;
+        n.w += q.w;
     }
+    o[0] = b.x + x[0] - c[0];
+    o[1] = b.y + x[1] - c[1];
+    o[2] = b.z + x[2] - c[2];
+    o[3] = b.w + x[3] - c[3];
+    t[0] = n.x;
+    t[1] = n.y;
+    t[2] = n.z;
+    t[3] = n.w;
 }
 
 // Centre-pass class of a Tersoff slot with m list neighbours: one thread
@@ -1217,7 +1288,7 @@ __device__ __noinline__ void check_lists(const DevParams& P, const HotParams<R>&
 
 // Atoms with at most REED_FAST_NB neighbours: everything in registers
 // (unrolled; missing neighbours have fc = P = Q = 0 and contribute nothing).
-template <typename R, int TT>
+template <typename R, int TT, bool TEAM>
 __device__ __forceinline__ R ters_centre_fast(const HotParams<R>& H, Win<R, TT>& W, int k, int m, int nact,
                                               unsigned& triplets)
 {
@@ -1310,7 +1381,7 @@ __device__ __forceinline__ R ters_centre_fast(const HotParams<R>& H, Win<R, TT>&
         az -= fz[p];
         if (p < m) {
             const unsigned s = W.need_map[idx[p]];
-            if (s < (unsigned)nact && rv[p] != (uint8_t)REED_NO_REV) W.bf_store((int)s, rv[p], fx[p], fy[p], fz[p]);
+            if (s < (unsigned)nact && rv[p] != (uint8_t)REED_NO_REV) W.template put_force<TEAM>((int)s, rv[p], fx[p], fy[p], fz[p]);
         }
     }
     if (k < nact) {
@@ -1319,24 +1390,27 @@ __device__ __forceinline__ R ters_centre_fast(const HotParams<R>& H, Win<R, TT>&
         f.y = ay;
         f.z = az;
         f.w = R(0);
-        W.frc[a] = f;
+        W.template put_centre<TEAM>(a, f);
     }
     return E;
 }
 
 // More than REED_FAST_NB neighbours (lists in shared memory or in an
-// overflow row): a group of G lanes per centre (G = 8, 16 or 32; lane l of
-// the group owns neighbours l and, for G = 32, l + 32).  The terms a lane
+// overflow row): a group of G lanes per centre (G = 8 or 16 with NH = 1, 32
+// with NH = 2; lane l of the group owns neighbours l and, for G = 32, l + 32).
+// The groups of 8 and of 16 run the same code, and its loops are not unrolled:
+// there is about one centre with more than eight neighbours in a step, and
+// what its warp would wait for is code that nothing else has brought into the
+// instruction cache.  The terms a lane
 // needs from the other neighbours are broadcast with shuffles inside the
 // group; sums over the group use the fixed butterfly order.  All 32 lanes of
 // the warp call it together, each group with its own slot k (k < 0: idle).
-template <typename R, int TT, int G>
-__device__ R ters_centre_group(const HotParams<R>& H, Win<R, TT>& W, int k, int nact, unsigned& triplets)
+template <typename R, int TT, int NH, bool TEAM>
+__device__ R ters_centre_group(const HotParams<R>& H, Win<R, TT>& W, const int G, int k, int nact, unsigned& triplets)
 {
-    constexpr int NH = G == 32 ? 2 : 1;
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, lg = lane & (G - 1);
-    const unsigned gmask = G == 32 ? FULL : (((1u << G) - 1u) << (lane & ~(G - 1)));
+    const unsigned gmask = NH == 2 ? FULL : (((1u << G) - 1u) << (lane & ~(G - 1)));
     const int m = k >= 0 ? (int)W.nnb[k] : 0;
     const int mmax = (int)__reduce_max_sync(FULL, (unsigned)m);
     int a = 0;
@@ -1380,6 +1454,7 @@ __device__ R ters_centre_group(const HotParams<R>& H, Win<R, TT>& W, int k, int 
     R zeta[NH];
 #pragma unroll
     for (int h = 0; h < NH; ++h) zeta[h] = R(0);
+#pragma unroll 1
     for (int p = 0; p < mmax; ++p) {
         const int src = p & (G - 1), hp = NH == 2 ? (p >> 5) : 0;
         const R vx = __shfl_sync(FULL, hp ? ux[NH - 1] : ux[0], src, G);
@@ -1409,6 +1484,7 @@ __device__ R ters_centre_group(const HotParams<R>& H, Win<R, TT>& W, int k, int 
     R sg[NH];
 #pragma unroll
     for (int h = 0; h < NH; ++h) sg[h] = R(0);
+#pragma unroll 1
     for (int j = 0; j < mmax; ++j) {
         const int src = j & (G - 1), hj = NH == 2 ? (j >> 5) : 0;
         const R vx = __shfl_sync(FULL, hj ? ux[NH - 1] : ux[0], src, G);
@@ -1442,11 +1518,12 @@ __device__ R ters_centre_group(const HotParams<R>& H, Win<R, TT>& W, int k, int 
         if (ok[h]) {
             const unsigned s = W.need_map[id[h]];
             const uint8_t e = rv[lg + G * h];
-            if (s < (unsigned)nact && e != (uint8_t)REED_NO_REV) W.bf_store((int)s, e, fx[h], fy[h], fz[h]);
+            if (s < (unsigned)nact && e != (uint8_t)REED_NO_REV) W.template put_force<TEAM>((int)s, e, fx[h], fy[h], fz[h]);
         }
     }
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) {
+    for (int o = NH == 2 ? 16 : 8; o > 0; o >>= 1) {
+        if (NH == 1 && o == 8 && G == 8) continue;
         ax += __shfl_xor_sync(FULL, ax, o);
         ay += __shfl_xor_sync(FULL, ay, o);
         az += __shfl_xor_sync(FULL, az, o);
@@ -1458,7 +1535,7 @@ __device__ R ters_centre_group(const HotParams<R>& H, Win<R, TT>& W, int k, int 
         f.y = ay;
         f.z = az;
         f.w = R(0);
-        W.frc[a] = f;
+        W.template put_centre<TEAM>(a, f);
     }
     return (lg == 0 && k >= 0) ? E : R(0);
 }
@@ -1469,28 +1546,33 @@ __device__ R ters_centre_group(const HotParams<R>& H, Win<R, TT>& W, int k, int 
 // of 8 lanes, four centres per warp), ncls[2] with up to 16 (two per warp)
 // and ncls[3] with more (one per warp).  The group tasks are dealt to the
 // warps from the last one down (the last warps have the fewest one-thread
-// slots).  Returns this thread's share of the Tersoff energy.
-template <typename R, int TT>
+// slots).  A team deals the tasks to the warps of all its CTAs, which are
+// numbered across the CTAs first.  Returns this thread's share of the Tersoff
+// energy.
+template <typename R, int TT, bool TEAM = false>
 __device__ R ters_centres(const HotParams<R>& H, Win<R, TT>& W, unsigned& triplets)
 {
     const int nact = W.S->active_count;
     const int n0 = W.S->ncls[0], n1 = W.S->ncls[1], n2 = W.S->ncls[2], n3 = W.S->ncls[3];
     R E = R(0);
-    for (int j = threadIdx.x; j < n0; j += blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    const int nw = TEAM ? (int)(blockDim.x >> 5) * W.team : (int)(blockDim.x >> 5);
+    const int w = TEAM ? (int)(threadIdx.x >> 5) * W.team + W.rank : (int)(threadIdx.x >> 5);
+#pragma unroll 1
+    for (int j = TEAM ? 32 * w + lane : (int)threadIdx.x; j < n0; j += TEAM ? 32 * nw : (int)blockDim.x) {
         const int k = W.order[j];
-        E += ters_centre_fast<R, TT>(H, W, k, W.nnb[k], nact, triplets);
+        E += ters_centre_fast<R, TT, TEAM>(H, W, k, W.nnb[k], nact, triplets);
     }
-    const int nw = blockDim.x >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int t1 = (n1 + 3) / 4, t2 = (n2 + 1) / 2, ntask = t1 + t2 + n3;
+#pragma unroll 1
     for (int t = nw - 1 - w; t < ntask; t += nw) {
-        if (t < t1) {
-            const int j = 4 * t + (lane >> 3);
-            E += ters_centre_group<R, TT, 8>(H, W, j < n1 ? (int)W.order[n0 + j] : -1, nact, triplets);
-        } else if (t < t1 + t2) {
-            const int j = 2 * (t - t1) + (lane >> 4);
-            E += ters_centre_group<R, TT, 16>(H, W, j < n2 ? (int)W.order[n0 + n1 + j] : -1, nact, triplets);
+        if (t < t1 + t2) {
+            const bool small = t < t1;
+            const int j = small ? 4 * t + (lane >> 3) : 2 * (t - t1) + (lane >> 4);
+            const int k = j < (small ? n1 : n2) ? (int)W.order[(small ? n0 : n0 + n1) + j] : -1;
+            E += ters_centre_group<R, TT, 1, TEAM>(H, W, small ? 8 : 16, k, nact, triplets);
         } else {
-            E += ters_centre_group<R, TT, 32>(H, W, (int)W.order[n0 + n1 + n2 + (t - t1 - t2)], nact, triplets);
+            E += ters_centre_group<R, TT, 2, TEAM>(H, W, 32, (int)W.order[n0 + n1 + n2 + (t - t1 - t2)], nact, triplets);
         }
     }
     return E;
@@ -1642,8 +1724,10 @@ __device__ void force_phase(const DevParams& P, const HotParams<R>& H, Win<R, TT
     } else {
         // integrated atoms through their slots, then every other present atom
         const int nact = W.S->active_count;
-        for (int k = threadIdx.x; k < nact; k += blockDim.x)
+    #pragma unroll 1
+    for (int k = threadIdx.x; k < nact; k += blockDim.x)
             atom_force<R, TT, KICK>(P, H, W, W.slot_atom[k], k, hdt, out, want_energy);
+        if (KICK && !W.S->near_frozen) return;
         for (int i = threadIdx.x; i < P.na; i += blockDim.x) {
             const V4<R> p = W.pos[i];
             if (!is_present(p)) continue;
@@ -1707,37 +1791,34 @@ __device__ __noinline__ void sum_ion_terms(const DevParams& P, TrackShared<R>* S
             }
         };
         for (int k = vw * 32 + lane; k < nact; k += vt) add(slot_atom[k]);
-        if (P.margin)
+        if (S->near_frozen)
             for (int i = vw * 32 + lane; i < P.na; i += vt) {
                 const V4<R> p = pos[i];
                 if (is_present(p) && !(is_active(p) && (unsigned)need_map[i] < (unsigned)nact)) add(i);
             }
-        fx = warp_sum(fx);
-        fy = warp_sum(fy);
-        fz = warp_sum(fz);
-        rho = warp_sum(rho);
-        if (lane == 0) {
-            R* row = S->red[vw];
-            row[0] = fx;
-            row[1] = fy;
-            row[2] = fz;
-            row[3] = rho;
-        }
+        const R s = warp_sum4(fx, fy, fz, rho);
+        if ((lane & 7) == 0) S->red[vw][lane >> 3] = s;
     }
 }
 
-// Block-reduce the partials into S->red row 0 (thread 0 reads them).
-template <typename R, int TT>
+// The partials of each warp into its row of S->red; the potential energy only
+// with ENERGY (a step does not need it).
+template <typename R, int TT, bool ENERGY = true>
 __device__ __forceinline__ void reduce_partials(Win<R, TT>& W, Partial<R>& q)
 {
+    constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    R fx = warp_sum(q.fx), fy = warp_sum(q.fy), fz = warp_sum(q.fz), rho = warp_sum(q.rho);
-    R vm = warp_max(q.vmax2), ep = warp_sum(q.epot), pm = warp_max(q.pmax);
-    int pr = warp_sum(q.pairs), bd = warp_sum(q.bonds);
+    R* row = W.S->red[wid];
+    const R s = warp_sum4(q.fx, q.fy, q.fz, q.rho);
+    if ((lane & 7) == 0) row[lane >> 3] = s;
+    const R vm = warp_max_pos(q.vmax2), pm = warp_max_pos(q.pmax), ep = ENERGY ? warp_sum(q.epot) : R(0);
+    const int pr = __reduce_add_sync(FULL, q.pairs), bd = __reduce_add_sync(FULL, q.bonds);
     if (lane == 0) {
-        R* row = W.S->red[wid];
-        row[0] = fx; row[1] = fy; row[2] = fz; row[3] = rho; row[4] = vm; row[5] = ep;
-        row[6] = R(pr); row[7] = R(bd); row[8] = pm;
+        row[4] = vm;
+        row[5] = ep;
+        row[6] = R(pr);
+        row[7] = R(bd);
+        row[8] = pm;
     }
 }
 
@@ -1878,7 +1959,6 @@ template <typename R> __device__ void launch_primary(const DevParams& P, IonStat
     I.vmax2 = R(0);
     I.pmax = R(0);
     I.t = 0.0;
-    I.e_elec = 0.0;
     I.steps = 0;
     I.level = 0;
     for (int d = 0; d < 3; ++d) I.A[d] = (int)floor(I.x[d] / P.a + P.anchor_shift);
@@ -1905,97 +1985,201 @@ template <typename R> __device__ void set_frame(const DevParams& P, TrackShared<
 
 // Electronic drag coefficient (Sec. 2 "Third"): F_e = -k v with
 // k = gamma (1 + s_loc (rho / rho0 - 1)) inside the target (z >= 0).
-template <typename R> __device__ __forceinline__ R drag_k(const HotParams<R>& H, const TrackShared<R>* S)
+template <typename R> __device__ __forceinline__ R drag_k(const HotParams<R>& H, R z, R zsurf, R rho)
 {
-    if (S->rel[2] < S->zsurf) return R(0);
-    return H.gamma * (R(1) + H.s_loc * (S->ion.rho * H.rho0_inv - R(1)));
+    if (z < zsurf) return R(0);
+    return H.gamma * (R(1) + H.s_loc * (rho * H.rho0_inv - R(1)));
 }
 
-// Prologue of a step (thread 0): dt from the fastest particle, ion half kick
-// and drift, window anchor check (Fig. "moving cell": the main cell follows
-// the ion).  FP64 work: the position and energy accumulations only.
-template <typename R> __device__ void ion_prologue(const DevParams& P, const HotParams<R>& H, TrackShared<R>* S)
+// Rare parts of ion_step, out of line: the code of a step runs through the
+// instruction cache once per step, and the ion's is run by a single warp.
+template <typename R> __device__ __noinline__ void set_frame_rare(const DevParams& P, TrackShared<R>* S)
 {
-    IonState<R>& I = S->ion;
-    const R v2 = I.v[0] * I.v[0] + I.v[1] * I.v[1] + I.v[2] * I.v[2];
-    const R vmax = sqrt(max(v2, I.vmax2));
-    R dt = H.dt_max;
-    if (vmax * dt > H.dx_max) dt = H.dx_max / vmax;
-    if (H.de_max > R(0)) {   // energy term: |dE_kin| <= de_max per step for every particle
-        const R pw = max(fabs(I.f[0] * I.v[0] + I.f[1] * I.v[1] + I.f[2] * I.v[2]), I.pmax);
-        if (pw * dt > H.de_max) {
-            dt = H.de_max / pw;
-            if (vmax * dt < H.dx_min) dt = H.dx_min / vmax;   // a step that moves nothing stalls
-        }
-    }
-    const R kd = drag_k<R>(H, S);
-    S->on1 = S->rel[2] >= S->zsurf;
-    const R h = R(0.5) * dt * H.invM1;
-    R de = R(0);
-    for (int d = 0; d < 3; ++d) {
-        const R fe = -kd * I.v[d];
-        de -= fe * I.v[d];
-        add_velocity<R>(I, d, h * (I.f[d] + fe));
-    }
-    I.e_elec += (double)(R(0.5) * dt * de);
-    int moved = 0;
-    for (int d = 0; d < 3; ++d) {
-        const R dx = dt * I.v[d];
-        I.x[d] += (double)dx;
-        S->rel[d] += dx;
-        S->Aold[d] = I.A[d];
-        // the ion leaves its anchor cell when rel leaves [-h a, (1-h) a)
-        if (S->rel[d] >= H.anchor_hi || S->rel[d] < H.anchor_lo) {
-            I.A[d] = (int)floor(I.x[d] / P.a + P.anchor_shift);
-            moved = 1;
-        }
-    }
-    if (moved) set_frame<R>(P, S);
-    S->shift = moved;
-    S->dt = dt;
+    set_frame<R>(P, S);
+    S->near_frozen = 0;   // (set again while the window moves)
 }
-
-// Epilogue (thread 0): ion second half kick, end and cloning checks.
-// Returns EV_NONE / EV_END / EV_CLONE; sets S->status and S->nclone.
-template <typename R>
-__device__ int ion_epilogue(const DevParams& P, const HotParams<R>& H, TrackShared<R>* S, const R red[REED_NRED])
+// the cloning depths that the track has just passed, on the FP64 depth
+template <typename R> __device__ __noinline__ int depths_passed(const DevParams& P, const TrackShared<R>* S)
 {
-    IonState<R>& I = S->ion;
-    const R dt = S->dt;
-    I.f[0] = red[0];
-    I.f[1] = red[1];
-    I.f[2] = red[2];
-    I.rho = red[3];
-    I.vmax2 = red[4];
-    I.pmax = red[8];
-    const R kd = drag_k<R>(H, S);
-    S->on2 = S->rel[2] >= S->zsurf;
-    const R h = R(0.5) * dt * H.invM1;
-    R de = R(0);
-    for (int d = 0; d < 3; ++d) {
-        const R fe = -kd * I.v[d];
-        de -= fe * I.v[d];
-        add_velocity<R>(I, d, h * (I.f[d] + fe));
-    }
-    I.e_elec += (double)(R(0.5) * dt * de);
-    I.t += (double)dt;
-    I.steps += 1;
-    const R E = R(0.5) * H.M1 * (I.v[0] * I.v[0] + I.v[1] * I.v[1] + I.v[2] * I.v[2]);
-    int st = 0;
-    if (!isfinite(E) || !isfinite(S->rel[0] + S->rel[1] + S->rel[2])) st = REED_TRACK_FAILED;
-    else if (E < H.e_stop) st = REED_TRACK_STOPPED;
-    else if (S->rel[2] < S->zback && I.v[2] < R(0)) st = REED_TRACK_BACKSCATTERED;
-    else if (I.steps >= P.step_cap) st = REED_TRACK_TRUNCATED;
-    S->status = st;
-    if (st) return EV_END;
+    const double z = track_depth(P, S->ion);
     int nc = 0;
-    if (S->rel[2] >= S->zthr) {
-        // passed one (or more) cloning depths: count them on the FP64 depth
-        const double z = track_depth(P, I);
-        while (I.level + nc < S->nthr && z >= S->thr[I.level + nc]) ++nc;
+    while (S->ion.level + nc < S->nthr && z >= S->thr[S->ion.level + nc]) ++nc;
+    return nc;
+}
+template <typename R>
+__device__ __noinline__ void trace_step(const DevParams& P, const DevBuf& B, const TrackShared<R>* S, double x, R v)
+{
+    const int lane = threadIdx.x & 31;
+    const size_t o = (size_t)S->pidx * P.trace_steps + (size_t)(S->ion.steps - 1);
+    if (lane < 4) B.trace[8 * o + lane] = x;
+    if (lane < 3) {
+        B.trace[8 * o + 4 + lane] = v;
+        B.trace_anchor[3 * o + lane] = S->ion.A[lane];
     }
-    S->nclone = nc;
-    return nc ? EV_CLONE : EV_NONE;
+    if (lane == 0) B.trace[8 * o + 7] = S->dt;
+}
+
+// The ion between two force passes (first warp; a barrier must precede and
+// follow): the sums over the atoms, the second half kick and the end and
+// cloning checks of the step (not with BEGIN, the start of a track), then the
+// next step's dt from the fastest particle, first half kick, drift and window
+// anchor check (Fig. "moving cell": the main cell follows the ion).  Returns
+// EV_NONE / EV_END / EV_CLONE (no next step prepared); sets S->event,
+// S->status and S->nclone.
+//
+// The rest of the CTA waits here, so what counts is the length of the chain.
+// Lanes 0-2 hold one component each and lane 3 the time: an FP64 addition
+// (some hundred cycles for the SM's FP64 unit) is issued twice a step and not
+// six times, and a column of the partial sums is added by one lane each.
+// `rows` warps left partial sums; those of the ion (columns 0-3) are in `vrows`
+// rows.
+template <typename R, bool BEGIN>
+__device__ __forceinline__ int ion_step(const DevParams& P, const DevBuf& B, const HotParams<R>& H, TrackShared<R>* S,
+                                        int rows, int vrows, bool tracing)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, c = min(lane, 2);
+    IonState<R>& I = S->ion;
+    __syncwarp();
+    R v = I.v[c], vlo = I.vlo[c], f = I.f[c], rho = I.rho, vmax2 = I.vmax2, pmax = I.pmax, dt = S->dt, rel = S->rel[c];
+    const R relz = S->rel[2], zsurf = S->zsurf;
+    double x = lane == 3 ? I.t : I.x[c];
+    // one half kick at the velocity the ion has (in these roundings on every
+    // path: a track's bits depend on them)
+    auto kick = [&]() {
+        const R kd = drag_k<R>(H, relz, zsurf, rho);
+        const R h = R(0.5) * dt * H.invM1;
+        add_velocity<R>(v, vlo, h * add_rn(f, mul_rn(-kd, v)));
+    };
+    int ev = EV_NONE;
+    if (!BEGIN) {
+        R acc = R(0);
+        const int col = min(lane, REED_NRED - 1), n = col < 4 ? vrows : rows;
+        const bool top = col == 4 || col == 8;
+        const R* q = &S->red[0][col];
+#pragma unroll 1
+        for (int w = 0; w < max(rows, vrows); w += 4, q += 4 * REED_NRED) {
+            const R y[4] = {q[0], q[REED_NRED], q[2 * REED_NRED], q[3 * REED_NRED]};
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (w + u < n) acc = top ? max(acc, y[u]) : acc + y[u];
+        }
+        f = acc;   // (of lanes 0-2)
+        rho = __shfl_sync(FULL, acc, 3);
+        vmax2 = __shfl_sync(FULL, acc, 4);
+        pmax = __shfl_sync(FULL, acc, 8);
+        // pairs and list entries (columns 6 and 7), and the phase clocks
+        if ((lane >= 6 && lane < 8) || (lane >= 16 && lane < 16 + PH_ADMIN)) {
+            const bool clk = lane >= 16;
+            static_assert(C_BONDS == C_PAIRS + 1, "counters of columns 6 and 7");
+            const int m = clk ? lane - 16 : 0;
+            S->cnt[clk ? C_PHASE0 + m : C_PAIRS + lane - 6] += clk ? S->mark[m + 1] - S->mark[m] : (unsigned)acc;
+        }
+        kick();
+        x += lane == 3 ? (double)dt : 0.0;
+        const long long steps = I.steps + 1;
+        const R v0 = __shfl_sync(FULL, v, 0), v1 = __shfl_sync(FULL, v, 1), v2 = __shfl_sync(FULL, v, 2);
+        const R E = R(0.5) * H.M1 * dist2(v0, v1, v2), far = S->rel[0] + S->rel[1] + relz;
+        if (lane == 0) {
+            S->mark[0] = S->mark[PH_FORCE + 1];
+            I.rho = rho;
+            I.vmax2 = vmax2;
+            I.pmax = pmax;
+            I.steps = steps;
+        }
+        if (lane < 3) I.f[lane] = f;
+        if (!(E >= H.e_stop) || !isfinite(E) || !isfinite(far) || (relz < S->zback && v2 < R(0)) || steps >= P.step_cap) {
+            int st = REED_TRACK_TRUNCATED;
+            if (!isfinite(E) || !isfinite(far)) st = REED_TRACK_FAILED;
+            else if (E < H.e_stop) st = REED_TRACK_STOPPED;
+            else if (relz < S->zback && v2 < R(0)) st = REED_TRACK_BACKSCATTERED;
+            if (lane == 0) S->status = st;
+            ev = EV_END;
+        }
+        if (tracing && steps <= P.trace_steps) {
+            __syncwarp();
+            trace_step<R>(P, B, S, x, v);
+        }
+        if (ev == EV_NONE && relz >= S->zthr) {
+            if (lane < 3) I.x[lane] = x;
+            __syncwarp();
+            const int nc = depths_passed<R>(P, S);
+            if (lane == 0) S->nclone = nc;
+            if (nc) ev = EV_CLONE;
+        }
+    }
+    bool moved = false;
+    if (ev == EV_NONE) {
+        const R v0 = __shfl_sync(FULL, v, 0), v1 = __shfl_sync(FULL, v, 1), v2 = __shfl_sync(FULL, v, 2);
+        const R vmax = sqrt(max(dist2(v0, v1, v2), vmax2));
+        dt = H.dt_max;
+        if (vmax * dt > H.dx_max) dt = H.dx_max / vmax;
+        if (H.de_max > R(0)) {   // energy term: |dE_kin| <= de_max per step for every particle
+            const R f0 = __shfl_sync(FULL, f, 0), f1 = __shfl_sync(FULL, f, 1), f2 = __shfl_sync(FULL, f, 2);
+            const R pw = max(fabs(f0 * v0 + f1 * v1 + f2 * v2), pmax);
+            if (pw * dt > H.de_max) {
+                dt = H.de_max / pw;
+                if (vmax * dt < H.dx_min) dt = H.dx_min / vmax;   // a step that moves nothing stalls
+            }
+        }
+        kick();
+        const R dx = dt * v;
+        rel += dx;
+        if (sizeof(R) == 8) x = fma((double)dt, lane < 3 ? (double)v : 0.0, x);
+        else x += lane < 3 ? (double)dx : 0.0;
+        if (lane < 3) S->rel[lane] = rel;
+        // the ion leaves its anchor cell when rel leaves [-h a, (1-h) a)
+        const bool out = lane < 3 && (rel >= H.anchor_hi || rel < H.anchor_lo);
+        moved = __any_sync(FULL, out);
+        if (moved && lane < 3) {
+            const int A = I.A[lane];
+            S->Aold[lane] = A;
+            if (out) I.A[lane] = (int)floor(x / P.a + P.anchor_shift);
+        }
+    }
+    if (lane < 3) {
+        I.v[lane] = v;
+        I.vlo[lane] = vlo;
+        I.x[lane] = x;
+    }
+    if (lane == 3) I.t = x;
+    if (lane == 0) {
+        S->event = ev;
+        S->dt = dt;
+        S->shift = moved;
+    }
+    if (moved) {
+        __syncwarp();
+        if (lane == 0) set_frame_rare<R>(P, S);
+    }
+    return ev;
+}
+template <typename R>
+__device__ __noinline__ void ion_begin(const DevParams& P, const DevBuf& B, TrackShared<R>* S)
+{
+    ion_step<R, true>(P, B, hot<R>(P), S, 0, 0, false);
+}
+
+// Work counters that follow from the list sizes, brought up to date before the
+// lists change (steps: the number completed; the current step's atoms have
+// moved, its centres have not been taken) and at the end of a track (thread 0).
+template <typename R> __device__ __forceinline__ void count_listed(TrackShared<R>* S, long long moved, long long centred)
+{
+    S->cnt[C_MOVED] += (unsigned long long)((moved - S->moved_from) * S->active_count);
+    for (int c = 0; c < 4; ++c)
+        S->cnt[C_CLS0 + c] += (unsigned long long)((centred - S->centred_from) * S->ncls[c]);
+    S->moved_from = moved;
+    S->centred_from = centred;
+}
+
+// Whether a frozen atom may come within the cutoff while the ion stays in the
+// anchor cell (it is there whenever forces are taken, see ion_step).
+template <typename R> __device__ __forceinline__ bool may_reach(const HotParams<R>& H, const V4<R>& p)
+{
+    const R dx = max(max(H.anchor_lo - p.x, p.x - H.anchor_hi), R(0));
+    const R dy = max(max(H.anchor_lo - p.y, p.y - H.anchor_hi), R(0));
+    const R dz = max(max(H.anchor_lo - p.z, p.z - H.anchor_hi), R(0));
+    return !(dx * dx + dy * dy + dz * dz > H.rc2 * R(1.01));
 }
 
 // Copy the window (pos, vel, frc) between shared memory and a clone record.
@@ -2092,6 +2276,97 @@ __device__ void initial_forces(const DevParams& P, const HotParams<R>& H, Win<R,
 
 #include "reed_adjoint.cuh"
 
+// First half kick and drift of one atom in a step; the two longest paths.
+template <typename R>
+__device__ __forceinline__ void move_atom(const HotParams<R>& H, const V4<R> f, R dt, R hdt, V4<R>& p, V4<R>& v,
+                                          R& pm1, R& pm2)
+{
+    const R k = hdt * of_species(H.invM2, p);
+    v.x += k * f.x;
+    v.y += k * f.y;
+    v.z += k * f.z;
+    const R sx = dt * v.x, sy = dt * v.y, sz = dt * v.z;
+    p.x += sx;
+    p.y += sy;
+    p.z += sz;
+    const R l2 = sx * sx + sy * sy + sz * sz;
+    if (l2 > R(0)) v.w += l2 * Mth<R>::rsqrt(l2);
+    pm2 = max(pm2, min(pm1, v.w));
+    pm1 = max(pm1, v.w);
+}
+
+// The parts of a step that run once in ten steps or less are out of line (the
+// step's own code is what the instruction cache should hold); they find the
+// window by themselves, so that the step's pointers stay in registers.
+#define REED_WINDOW(W, P, B)                                                                                   \
+    extern __shared__ __align__(16) unsigned char smem[];                                                      \
+    Win<R, TT> W(smem, P.na, P.bond_cap, 0, P.g_nbins, P.act_cap,                                              \
+                 B.spill ? B.spill + (size_t)blockIdx.x * B.spill_stride : nullptr)
+
+// Phase A of a step that moves the window.
+template <typename R, int TT>
+__device__ __noinline__ void move_window(const DevParams& P, const DevBuf& B, R dt, R hdt, bool lead)
+{
+    REED_WINDOW(W, P, B);
+    TrackShared<R>* S = W.S;
+    const HotParams<R>& H = hot<R>(P);
+    const uint64_t key = S->ion.key;
+    R pm1 = R(0), pm2 = R(0);
+    for (int i = threadIdx.x; i < P.na; i += blockDim.x) {
+        V4<R> p = W.pos[i], v = W.vel[i], f = W.frc[i];
+        if (is_active(p)) move_atom<R>(H, f, dt, hdt, p, v, pm1, pm2);
+        const V4<R> p0 = p, v0 = v;
+        if (reanchor_atom<R>(P, H, key, i, S->Aold, S->ion.A, p, v, f) && lead)
+            deposit_damage<R>(P, B, p0, v0, S->Aold, ldexp(1.0, -S->ion.level));
+        W.pos[i] = p;
+        W.vel[i] = v;
+        W.frc[i] = f;
+        if (is_present(p) && !is_active(p) && may_reach<R>(H, p)) S->near_frozen = 1;
+    }
+}
+
+// New lists in a step (ends with a barrier): a refresh where that is enough
+// (not after a window move), else a build.  Returns the entries and list rows
+// that did not fit.
+template <typename R, int TT>
+__device__ __noinline__ int2 renew_lists(const DevParams& P, const DevBuf& B, bool shift)
+{
+    REED_WINDOW(W, P, B);
+    TrackShared<R>* S = W.S;
+    const HotParams<R>& H = hot<R>(P);
+    int nbovf = 0, capovf = 0;
+    bool refreshed = false;
+    if (threadIdx.x == 0) count_listed<R>(S, S->ion.steps + 1, S->ion.steps);
+    if constexpr (TT == REED_TT_TERSOFF) {
+        if (!shift) refreshed = refresh_lists<R, TT>(P, H, W, nbovf);
+    }
+    if (!refreshed) build_neighbours<R, TT>(P, H, W, nbovf, capovf);
+    __syncthreads();
+    if (threadIdx.x == 0) ++S->cnt[refreshed ? C_REFRESH : C_REBUILDS];
+    if (P.nl_check) check_lists<R, TT>(P, H, W, refreshed ? H.tcut * H.tcut : H.rlist2);
+    return make_int2(nbovf, capovf);
+}
+
+// The start of a track: the lists and, of a primary, the forces (a barrier
+// must precede; ends with one).  Returns the entries and list rows that did
+// not fit and this thread's bond-angle terms.
+template <typename R, int TT>
+__device__ __noinline__ int3 start_track(const DevParams& P, const DevBuf& B, bool forces, int vt)
+{
+    REED_WINDOW(W, P, B);
+    const HotParams<R>& H = hot<R>(P);
+    int nbovf = 0, capovf = 0;
+    unsigned triplets = 0;
+    if (forces) {
+        initial_forces<R, TT>(P, H, W, nbovf, capovf, triplets, vt);
+    } else {
+        build_neighbours<R, TT>(P, H, W, nbovf, capovf);
+        if (threadIdx.x == 0) ++W.S->cnt[C_REBUILDS];
+        __syncthreads();
+    }
+    return make_int3(nbovf, capovf, (int)triplets);
+}
+
 // ---------------------------------------------------------------------------
 // The persistent kernel of the models with target-target forces (the
 // ion-target-only model and its adjoint: reed_ion.cuh).
@@ -2099,6 +2374,7 @@ __device__ void initial_forces(const DevParams& P, const HotParams<R>& H, Win<R,
 // the workloads allows, so registers are budgeted for that occupancy.
 // ---------------------------------------------------------------------------
 template <typename R, int TT> constexpr int track_min_ctas() { return TT == REED_TT_TERSOFF && sizeof(R) == 4 ? 2 : 1; }
+
 
 // Threads of a track's CTA at most.  The pair-list model: one track fills an
 // SM's shared memory, so its warps are all that the SM gets -- 24 of them, one
@@ -2111,14 +2387,28 @@ template <typename R, int TT> constexpr int track_max_threads()
 // Threads of a CTA whose run sums by vt virtual threads.
 template <typename R, int TT> inline int track_threads(int act_cap)
 {
-    if (TT == REED_TT_TERSOFF) return 256;
     const int t = (act_cap + 31) / 32 * 32;
     return t < 256 ? 256 : (t > track_max_threads<R, TT>() ? track_max_threads<R, TT>() : t);
 }
 
-template <typename R, int TT>
-__global__ void __launch_bounds__((track_max_threads<R, TT>()), (track_min_ctas<R, TT>())) reed_track_kernel(
-    const __grid_constant__ DevParams P, const __grid_constant__ DevBuf B, const int vt)
+// TEAM: the CTAs of a cluster follow one track together (launched without
+// cloning, a cluster per primary).  Each keeps the whole window and makes the
+// same lists, moves and kicks; the Tersoff centres, most of a step's
+// arithmetic, are shared out, each result going into every CTA's window
+// through distributed shared memory.  CTA 0 leads: it alone takes tracks,
+// updates the ion, and tallies.  The others follow its decisions, so that all
+// pass the same cluster barriers.  61 As tracks in FP64, bound by the SMs' FP64
+// pipes: 361 -> 213 ms with teams of two; 37 in the mixed form (512 threads
+// alone on an SM: 46 ms; 256: 52 ms): 35 ms.
+//
+// Much of a step's time is instruction fetch: the code of one step (centres 19
+// + 35 KB, ion 9 KB, lists) goes through the instruction cache once per step,
+// and a warp that runs alone waits for each line of it.  So the rare parts are
+// calls (REED_WINDOW), short loops are not unrolled, and the groups of 8 and 16
+// lanes share their code: 4096 As ions of 10 keV 1139 -> 977 ms.
+template <typename R, int TT, int MAX_THREADS = track_max_threads<R, TT>(), bool TEAM = false>
+__global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : track_min_ctas<R, TT>()))
+    reed_track_kernel(const __grid_constant__ DevParams P, const __grid_constant__ DevBuf B, const int vt)
 {
     static_assert(TT != REED_TT_NONE, "the ion-target-only model has its own kernel");
     extern __shared__ __align__(16) unsigned char smem[];
@@ -2127,11 +2417,37 @@ __global__ void __launch_bounds__((track_max_threads<R, TT>()), (track_min_ctas<
     TrackShared<R>* S = W.S;
     const HotParams<R>& H = hot<R>(P);
     const int tid = threadIdx.x;
+    if (TEAM) {
+        W.team = cluster_size();
+        W.rank = cluster_rank();
+        W.sp_step = (long long)B.spill_stride;
+    }
+    const bool lead = !TEAM || W.rank == 0;
+    // after a cluster barrier: the leader's track and ion state
+    auto follow = [&]() {
+        if (!TEAM || lead) return;
+        static_assert(offsetof(TrackShared<R>, thr) % sizeof(uint2) == 0, "copied in 8-byte words");
+        const uint2* from = reinterpret_cast<const uint2*>(in_cta(S, 0));
+        uint2* to = reinterpret_cast<uint2*>(S);
+        for (int k = tid; k < (int)(offsetof(TrackShared<R>, thr) / sizeof(uint2)); k += blockDim.x) to[k] = from[k];
+        __syncthreads();
+    };
+    auto team_sync = [&]() {
+        if (TEAM) cluster_sync();
+        else __syncthreads();
+    };
     unsigned char* stack = B.stacks ? B.stacks + (size_t)blockIdx.x * B.stack_stride : nullptr;
 
     int nbovf = 0, capovf = 0;
     unsigned triplets = 0;   // bond-angle terms of this thread in the current track
-    // phase clocks (thread 0): time between consecutive barriers of a step
+    // phase clocks (thread 0): the end of phases p .. PH_FORCE of a step (a later
+    // phase overwrites its own; ion_step adds them up), and whole laps outside
+    auto mark = [&](int p) {
+        if (tid == 0) {
+            const unsigned now = (unsigned)clock64();
+            for (; p <= PH_FORCE; ++p) S->mark[p + 1] = now;
+        }
+    };
     auto lap = [&](int phase) {
         if (tid == 0) {
             const long long now = clock64();
@@ -2143,12 +2459,14 @@ __global__ void __launch_bounds__((track_max_threads<R, TT>()), (track_min_ctas<
         S->top = 0;
         S->t_mark = clock64();
         for (int c = 0; c < REED_NCOUNT; ++c) S->cnt[c] = 0;
+        for (int c = 0; c < 4; ++c) S->ncls[c] = 0;   // (stays so without Tersoff lists)
     }
     W.clear_grid(P);
 
     for (;;) {
         // ---- acquire a track: own clone stack first, then a new primary
-        if (tid == 0) {
+        if (tid == 0) S->near_frozen = P.margin ? 1 : 0;   // (until the first window move)
+        if (lead && tid == 0) {
             S->nthr = P.nthr;
             for (int k = 0; k < P.nthr; ++k) S->thr[k] = P.thr_from_device ? B.thr[k] : P.thr[k];
             if (S->top > 0) {
@@ -2189,7 +2507,8 @@ __global__ void __launch_bounds__((track_max_threads<R, TT>()), (track_min_ctas<
                 }
             }
         }
-        __syncthreads();
+        team_sync();
+        follow();
         const int src = S->src;
         if (src == SRC_NONE) break;
         if (src == SRC_PRIMARY) {
@@ -2210,7 +2529,6 @@ __global__ void __launch_bounds__((track_max_threads<R, TT>()), (track_min_ctas<
                 W.frc[i] = f;
             }
             __syncthreads();
-            initial_forces<R, TT>(P, H, W, nbovf, capovf, triplets, vt);
         } else if (src == SRC_STOLEN) {
             const unsigned char* rec = B.pool + (size_t)S->slot * B.entry_bytes;
             if (tid == 0) {
@@ -2228,9 +2546,6 @@ __global__ void __launch_bounds__((track_max_threads<R, TT>()), (track_min_ctas<
                 atomicSub(&B.pool_ctl[1], 1u);
                 if (B.splits) atomicAdd(&B.splits[REED_MAX_THR], 1ull);
             }
-            build_neighbours<R, TT>(P, H, W, nbovf, capovf);
-            if (tid == 0) ++S->cnt[C_REBUILDS];
-            __syncthreads();
         } else {
             unsigned char* rec = stack + (size_t)(S->top - 1) * B.entry_bytes;
             if (tid == 0) {
@@ -2240,64 +2555,51 @@ __global__ void __launch_bounds__((track_max_threads<R, TT>()), (track_min_ctas<
             copy_window<R, TT>(P, W, rec, false);
             __syncthreads();
             if (tid == 0) S->top -= 1;
-            build_neighbours<R, TT>(P, H, W, nbovf, capovf);
-            if (tid == 0) ++S->cnt[C_REBUILDS];
-            __syncthreads();
+        }
+        {
+            const int3 n = start_track<R, TT>(P, B, src == SRC_PRIMARY, vt);
+            nbovf += n.x;
+            capovf += n.y;
+            if (lead) triplets += (unsigned)n.z;   // (of a team, counted by the leader)
         }
         const bool tracing = (src == SRC_PRIMARY) && (S->pidx < P.trace_tracks);
-        const long long pidx = S->pidx;
 
         // ---- step loop
-        bool need_prologue = true;
         lap(PH_ADMIN);
+        if (tid == 0) {
+            S->mark[0] = (unsigned)S->t_mark;
+            S->moved_from = S->centred_from = S->steps_from = S->ion.steps;
+        }
+        bool need_prologue = true;
         for (;;) {
             if (need_prologue) {
-                if (tid == 0) ion_prologue<R>(P, H, S);
-                __syncthreads();
-                lap(PH_ION);
+                if (lead && tid < 32) ion_begin<R>(P, B, S);
+                team_sync();
+                follow();
             }
+            mark(PH_ION);
             const R dt = R(S->dt), hdt = R(0.5) * R(S->dt);
             const int shift = S->shift;
-            const uint64_t key = S->ion.key;
             Partial<R> q = {R(0), R(0), R(0), R(0), R(0), R(0), 0, 0};
             // phase A: first half kick + drift of the atoms integrated before
             // the window moves, then the move (a step's kick and drift precede
             // its window update: an atom entering the integrated region is
             // first kicked at the end of this step, one leaving it still
-            // moves in this step)
+            // moves in this step).  Frozen atoms do not move; the others have
+            // list slots.
             R pm1 = R(0), pm2 = R(0);   // this thread's two longest paths
-            if (tid == 0) S->cnt[C_MOVED] += (unsigned)S->active_count;
-            for (int i = tid; i < P.na; i += blockDim.x) {
-                V4<R> p = W.pos[i];
-                const bool act = is_active(p);
-                if (!act && !shift) continue;   // frozen atoms do not move
-                V4<R> v = W.vel[i], f = W.frc[i];
-                if (act) {
-                    const R k = hdt * H.invM2[species_of(p)];
-                    v.x += k * f.x;
-                    v.y += k * f.y;
-                    v.z += k * f.z;
-                    const R sx = dt * v.x, sy = dt * v.y, sz = dt * v.z;
-                    p.x += sx;
-                    p.y += sy;
-                    p.z += sz;
-                    const R l2 = sx * sx + sy * sy + sz * sz;
-                    if (l2 > R(0)) v.w += l2 * Mth<R>::rsqrt(l2);
-                    if (v.w > pm1) {
-                        pm2 = pm1;
-                        pm1 = v.w;
-                    } else if (v.w > pm2) {
-                        pm2 = v.w;
-                    }
+            if (!shift) {
+#pragma unroll 1
+                for (int k = tid; k < S->active_count; k += blockDim.x) {
+                    const int i = W.slot_atom[k];
+                    V4<R> p = W.pos[i], v = W.vel[i];
+                    move_atom<R>(H, W.frc[i], dt, hdt, p, v, pm1, pm2);
+                    W.pos[i] = p;
+                    W.vel[i] = v;
                 }
-                if (shift) {
-                    const V4<R> p0 = p, v0 = v;
-                    if (reanchor_atom<R>(P, H, key, i, S->Aold, S->ion.A, p, v, f))
-                        deposit_damage<R>(P, B, p0, v0, S->Aold, ldexp(1.0, -S->ion.level));
-                }
-                W.pos[i] = p;
-                W.vel[i] = v;
-                if (shift) W.frc[i] = f;
+            } else {
+                move_window<R, TT>(P, B, dt, hdt, lead);   // (lists are rebuilt: no paths)
+                if (tid == 0) ++S->cnt[C_SHIFTS];
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
@@ -2310,7 +2612,7 @@ __global__ void __launch_bounds__((track_max_threads<R, TT>()), (track_min_ctas<
                 S->path2[tid >> 5][1] = pm2;
             }
             __syncthreads();
-            lap(PH_MOVE);
+            mark(PH_MOVE);
             // every thread merges the per-warp pairs in the same order
             R m1 = R(0), m2 = R(0);
             for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
@@ -2319,54 +2621,29 @@ __global__ void __launch_bounds__((track_max_threads<R, TT>()), (track_min_ctas<
                 m1 = fmax(m1, q1);
             }
             if (shift || m1 + m2 > H.skin) {
-                bool refreshed = false;
-                if constexpr (TT == REED_TT_TERSOFF) {
-                    if (!shift) refreshed = refresh_lists<R, TT>(P, H, W, nbovf);
-                }
-                if (!refreshed) build_neighbours<R, TT>(P, H, W, nbovf, capovf);
-                __syncthreads();
-                if (tid == 0) ++S->cnt[refreshed ? C_REFRESH : C_REBUILDS];
-                if (P.nl_check)
-                    check_lists<R, TT>(P, H, W, refreshed ? H.tcut * H.tcut : H.rlist2);
-                lap(PH_BUILD);
+                const int2 n = renew_lists<R, TT>(P, B, shift);
+                nbovf += n.x;
+                capovf += n.y;
+                mark(PH_BUILD);
             }
             if constexpr (TT == REED_TT_TERSOFF) {
-                ters_centres<R, TT>(H, W, triplets);
-                __syncthreads();
-                lap(PH_PASS1);
-                if (tid == 0)
-                    for (int c = 0; c < 4; ++c) S->cnt[C_CLS0 + c] += (unsigned)S->ncls[c];
+                // (every CTA of a team has read its force rows of the last step)
+                if (TEAM) cluster_sync();
+                ters_centres<R, TT, TEAM>(H, W, triplets);
+                team_sync();
+                mark(PH_PASS1);
             }
             force_phase<R, TT, true>(P, H, W, hdt, q, false);
-            reduce_partials<R, TT>(W, q);
+            reduce_partials<R, TT, false>(W, q);
             __syncthreads();
-            if (vt != (int)blockDim.x) {
+            if (lead && vt != (int)blockDim.x) {
                 sum_ion_terms<R>(P, W.S, W.pos, W.frc, W.slot_atom, W.need_map, vt);
                 __syncthreads();
             }
-            lap(PH_FORCE);
-            if (tid == 0) {
-                R red[REED_NRED];
-                gather_partials<R, TT>(W, red, vt >> 5);
-                S->cnt[C_PAIRS] += (unsigned long long)red[6];
-                S->cnt[C_BONDS] += (unsigned long long)red[7];
-                S->cnt[C_SHIFTS] += (unsigned)shift;
-                ++S->cnt[C_STEPS];
-                int ev = ion_epilogue<R>(P, H, S, red);
-                if (tracing && S->ion.steps <= P.trace_steps) {
-                    const IonState<R>& I = S->ion;
-                    size_t o = (size_t)pidx * P.trace_steps + (size_t)(I.steps - 1);
-                    double* t8 = B.trace + 8 * o;
-                    t8[0] = I.x[0]; t8[1] = I.x[1]; t8[2] = I.x[2]; t8[3] = I.t;
-                    t8[4] = I.v[0]; t8[5] = I.v[1]; t8[6] = I.v[2]; t8[7] = S->dt;
-                    int* a3 = B.trace_anchor + 3 * o;
-                    a3[0] = I.A[0]; a3[1] = I.A[1]; a3[2] = I.A[2];
-                }
-                S->event = ev;
-                if (ev == EV_NONE) ion_prologue<R>(P, H, S);
-            }
-            __syncthreads();
-            lap(PH_ION);
+            mark(PH_FORCE);
+            if (lead && tid < 32) ion_step<R, false>(P, B, H, S, (int)blockDim.x >> 5, vt >> 5, tracing);
+            team_sync();
+            follow();
             const int ev = S->event;
             if (ev == EV_NONE) {
                 need_prologue = false;
@@ -2442,17 +2719,20 @@ __global__ void __launch_bounds__((track_max_threads<R, TT>()), (track_min_ctas<
             __syncthreads();
         }
         // ---- track finished
-        lap(PH_ADMIN);
-        if (B.damage) {
+        if (tid == 0) {
+            S->t_mark = clock64();
+            count_listed<R>(S, S->ion.steps, S->ion.steps);
+            S->cnt[C_STEPS] += (unsigned long long)(S->ion.steps - S->steps_from);
+        }
+        if (B.damage && lead) {
             const int A[3] = {S->ion.A[0], S->ion.A[1], S->ion.A[2]};
             const double wgt = ldexp(1.0, -S->ion.level);
             for (int i = tid; i < P.na; i += blockDim.x) {
                 const V4<R> p = W.pos[i];
                 if (is_active(p)) deposit_damage<R>(P, B, p, W.vel[i], A, wgt);
             }
-            __syncthreads();
         }
-        if (tid == 0) {
+        if (lead && tid == 0) {
             if (S->status == REED_TRACK_FAILED) {
                 ++S->cnt[C_FAILED];
                 atomicOr(B.status, ERR_NONFINITE);
@@ -2467,6 +2747,7 @@ __global__ void __launch_bounds__((track_max_threads<R, TT>()), (track_min_ctas<
         }
         __syncthreads();
     }
+    if (TEAM) cluster_sync();   // (a follower may still be reading the leader's state)
     if (nbovf || capovf) atomicOr(B.status, ERR_NEIGHBOR);
     // flush counters
     int ov = nbovf, oc = capovf;
@@ -2474,11 +2755,11 @@ __global__ void __launch_bounds__((track_max_threads<R, TT>()), (track_min_ctas<
         ov += __shfl_xor_sync(0xffffffffu, ov, o);
         oc += __shfl_xor_sync(0xffffffffu, oc, o);
     }
-    if ((tid & 31) == 0 && ov) atomicAdd(&B.counters[C_NBOVF], (unsigned long long)ov);
-    if ((tid & 31) == 0 && oc) atomicAdd(&B.counters[C_CAPOVF], (unsigned long long)oc);
+    if ((tid & 31) == 0 && ov && lead) atomicAdd(&B.counters[C_NBOVF], (unsigned long long)ov);
+    if ((tid & 31) == 0 && oc && lead) atomicAdd(&B.counters[C_CAPOVF], (unsigned long long)oc);
     __syncthreads();
     lap(PH_ADMIN);
     __syncthreads();
     for (int c = tid; c < REED_NCOUNT; c += blockDim.x)
-        if (S->cnt[c]) atomicAdd(&B.counters[c], S->cnt[c]);
+        if (S->cnt[c] && (lead || c == C_TRIPLETS)) atomicAdd(&B.counters[c], S->cnt[c]);
 }

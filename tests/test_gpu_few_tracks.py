@@ -1,0 +1,62 @@
+"""A run with no more tracks than SMs (or other processors' worth of CTAs) is
+launched in another shape than a large batch: every track must come out the
+same, bit for bit, for each number of tracks around the places where the shape
+changes.
+"""
+import numpy as np
+import pytest
+
+from paper_0810_4737_gb300.workloads import workload
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def R():
+    from paper_0810_4737_gb300 import build, reed
+    build.build()
+    return reed
+
+
+def _records(R, w, n, prec, **kw):
+    with R.Reed(w) as ctx:
+        ctx.run(n_ions=n, seed=11, precision=prec, **kw)
+        rec = ctx.records()
+        st = ctx.stats()
+        damage = ctx.damage_map() if ctx.w["damage_n"] else None
+    return rec[np.argsort(rec["id"], kind="stable")], st, damage
+
+
+@pytest.mark.parametrize("name,prec,steps,few", [
+    ("as10kev_si_300k_tersoff", 0, 400, (1, 5, 76, 152, 153, 304)),
+    ("as10kev_si_300k_tersoff", 1, 120, (1, 5, 20, 39, 77, 152)),
+    ("ar30kev_ceo2_300k_buck", 0, 150, (1, 5, 39, 77, 152)),
+    ("ar30kev_ceo2_300k_buck", 1, 40, (1, 5, 77)),
+    ("b1kev_si_0k_zbl", 0, 500, (1, 5, 153)),
+    ("b1kev_si_0k_zbl", 1, 200, (1, 153))])
+def test_tracks_do_not_depend_on_the_launch_shape(R, name, prec, steps, few):
+    w = workload(name, thresholds=[], step_cap=steps)
+    ref, _, _ = _records(R, w, 330, prec)
+    for n in few:
+        rec, st, _ = _records(R, w, n, prec)
+        assert st["tracks"] == st["primaries"] == n
+        assert rec.tobytes() == ref[:n].tobytes(), n
+
+
+def test_low_energy_tracks_to_their_end(R):
+    """Whole tracks with window moves, cascades and list refreshes."""
+    w = workload("as10kev_si_300k_tersoff", thresholds=[], energy=300.0)
+    ref, _, _ = _records(R, w, 200, 0)
+    rec, _, _ = _records(R, w, 9, 0)
+    assert rec.tobytes() == ref[:9].tobytes()
+    w = workload("as10kev_si_300k_tersoff", thresholds=[], energy=60.0)
+    ref, _, _ = _records(R, w, 160, 1)
+    rec, _, _ = _records(R, w, 9, 1)
+    assert rec.tobytes() == ref[:9].tobytes()
+
+
+def test_damage_of_a_single_track_is_deposited_once(R):
+    w = workload("ar30kev_ceo2_300k_buck", thresholds=[], energy=1000.0, step_cap=400)
+    a, _, da = _records(R, w, 1, 0)
+    b, _, db = _records(R, w, 1, 0, ctas_per_sm=1)
+    assert a.tobytes() == b.tobytes() and np.allclose(da[0], db[0], rtol=1e-12, atol=0)
