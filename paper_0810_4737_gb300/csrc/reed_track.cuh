@@ -74,7 +74,6 @@ template <typename R> struct TrackShared {
     long long rec_index;
     R xbi[3], vbi[3], ubi[3], vh[3], irel[3], vub, k1;
     double gth[8];
-    R adj_red[REED_ADJ_WARPS][12];
     int near_frozen;      // a frozen atom may come within the cutoff of the ion before the next window move
     unsigned mark[6];     // clocks: the end of the last step's forces, then of each phase of this step
     long long moved_from, centred_from, steps_from;   // see count_listed; steps before this CTA took the track
@@ -90,7 +89,10 @@ template <typename R> struct TrackShared {
     int nstale, nhot;
     uint16_t stale[REED_MAX_STALE];
     uint16_t hot[REED_MAX_HOT];
-    alignas(16) int scan[REED_MAX_WARPS][4];
+    union {               // (list builds; the adjoint has none)
+        alignas(16) int scan[REED_MAX_WARPS][4];
+        R adj_red[REED_ADJ_WARPS][12];
+    };
     R red[REED_MAX_WARPS][REED_NRED];
     R path2[REED_MAX_WARPS][2];   // per warp: the two longest atom paths since the list build
 };
@@ -1991,6 +1993,7 @@ template <typename R> __device__ __forceinline__ R drag_k(const HotParams<R>& H,
     return H.gamma * (R(1) + H.s_loc * (rho * H.rho0_inv - R(1)));
 }
 
+#define REED_RARE(x) __builtin_expect(!!(x), 0)   // (its code is laid out behind the step's)
 // Rare parts of ion_step, out of line: the code of a step runs through the
 // instruction cache once per step, and the ion's is run by a single warp.
 template <typename R> __device__ __noinline__ void set_frame_rare(const DevParams& P, TrackShared<R>* S)
@@ -2062,33 +2065,29 @@ __device__ __forceinline__ int ion_step(const DevParams& P, const DevBuf& B, con
             const R y[4] = {q[0], q[REED_NRED], q[2 * REED_NRED], q[3 * REED_NRED]};
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-                if (w + u < n) acc = top ? max(acc, y[u]) : acc + y[u];
+            {
+                const R sum = acc + y[u], big = max(acc, y[u]), next = top ? big : sum;
+                acc = w + u < n ? next : acc;
+            }
         }
         f = acc;   // (of lanes 0-2)
         rho = __shfl_sync(FULL, acc, 3);
         vmax2 = __shfl_sync(FULL, acc, 4);
         pmax = __shfl_sync(FULL, acc, 8);
-        // pairs and list entries (columns 6 and 7), and the phase clocks
-        if ((lane >= 6 && lane < 8) || (lane >= 16 && lane < 16 + PH_ADMIN)) {
-            const bool clk = lane >= 16;
-            static_assert(C_BONDS == C_PAIRS + 1, "counters of columns 6 and 7");
-            const int m = clk ? lane - 16 : 0;
-            S->cnt[clk ? C_PHASE0 + m : C_PAIRS + lane - 6] += clk ? S->mark[m + 1] - S->mark[m] : (unsigned)acc;
-        }
         kick();
         x += lane == 3 ? (double)dt : 0.0;
         const long long steps = I.steps + 1;
         const R v0 = __shfl_sync(FULL, v, 0), v1 = __shfl_sync(FULL, v, 1), v2 = __shfl_sync(FULL, v, 2);
         const R E = R(0.5) * H.M1 * dist2(v0, v1, v2), far = S->rel[0] + S->rel[1] + relz;
         if (lane == 0) {
-            S->mark[0] = S->mark[PH_FORCE + 1];
             I.rho = rho;
             I.vmax2 = vmax2;
             I.pmax = pmax;
             I.steps = steps;
         }
         if (lane < 3) I.f[lane] = f;
-        if (!(E >= H.e_stop) || !isfinite(E) || !isfinite(far) || (relz < S->zback && v2 < R(0)) || steps >= P.step_cap) {
+        if (REED_RARE(!(E >= H.e_stop) || !isfinite(E) || !isfinite(far) || (relz < S->zback && v2 < R(0)) ||
+                      steps >= P.step_cap)) {
             int st = REED_TRACK_TRUNCATED;
             if (!isfinite(E) || !isfinite(far)) st = REED_TRACK_FAILED;
             else if (E < H.e_stop) st = REED_TRACK_STOPPED;
@@ -2096,11 +2095,11 @@ __device__ __forceinline__ int ion_step(const DevParams& P, const DevBuf& B, con
             if (lane == 0) S->status = st;
             ev = EV_END;
         }
-        if (tracing && steps <= P.trace_steps) {
+        if (REED_RARE(tracing && steps <= P.trace_steps)) {
             __syncwarp();
             trace_step<R>(P, B, S, x, v);
         }
-        if (ev == EV_NONE && relz >= S->zthr) {
+        if (REED_RARE(ev == EV_NONE && relz >= S->zthr)) {
             if (lane < 3) I.x[lane] = x;
             __syncwarp();
             const int nc = depths_passed<R>(P, S);
@@ -2131,7 +2130,7 @@ __device__ __forceinline__ int ion_step(const DevParams& P, const DevBuf& B, con
         // the ion leaves its anchor cell when rel leaves [-h a, (1-h) a)
         const bool out = lane < 3 && (rel >= H.anchor_hi || rel < H.anchor_lo);
         moved = __any_sync(FULL, out);
-        if (moved && lane < 3) {
+        if (REED_RARE(moved) && lane < 3) {
             const int A = I.A[lane];
             S->Aold[lane] = A;
             if (out) I.A[lane] = (int)floor(x / P.a + P.anchor_shift);
@@ -2148,11 +2147,29 @@ __device__ __forceinline__ int ion_step(const DevParams& P, const DevBuf& B, con
         S->dt = dt;
         S->shift = moved;
     }
-    if (moved) {
+    if (REED_RARE(moved)) {
         __syncwarp();
         if (lane == 0) set_frame_rare<R>(P, S);
     }
     return ev;
+}
+// Meanwhile the second warp adds up the step's pairs and list entries (columns
+// 6 and 7 of the partial sums) and its phase clocks, which its first lane took.
+template <typename R> __device__ __forceinline__ void count_step(TrackShared<R>* S, int rows)
+{
+    static_assert(C_BONDS == C_PAIRS + 1, "counters of columns 6 and 7");
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    unsigned add = 0;
+    if (lane < 2) {
+#pragma unroll 4
+        for (int w = 0; w < rows; ++w) add += (unsigned)S->red[w][6 + lane];
+    } else if (lane < 2 + PH_ADMIN) {
+        add = S->mark[lane - 1] - S->mark[lane - 2];
+    }
+    if (lane < 2 + PH_ADMIN) S->cnt[lane < 2 ? C_PAIRS + lane : C_PHASE0 + lane - 2] += add;
+    __syncwarp();
+    if (lane == 0) S->mark[0] = S->mark[PH_FORCE + 1];
 }
 template <typename R>
 __device__ __noinline__ void ion_begin(const DevParams& P, const DevBuf& B, TrackShared<R>* S)
@@ -2440,10 +2457,10 @@ __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : t
 
     int nbovf = 0, capovf = 0;
     unsigned triplets = 0;   // bond-angle terms of this thread in the current track
-    // phase clocks (thread 0): the end of phases p .. PH_FORCE of a step (a later
-    // phase overwrites its own; ion_step adds them up), and whole laps outside
+    // phase clocks: the end of phases p .. PH_FORCE of a step (a later phase
+    // overwrites its own; count_step adds them up), and whole laps outside
     auto mark = [&](int p) {
-        if (tid == 0) {
+        if (tid == 32) {
             const unsigned now = (unsigned)clock64();
             for (; p <= PH_FORCE; ++p) S->mark[p + 1] = now;
         }
@@ -2588,7 +2605,7 @@ __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : t
             // moves in this step).  Frozen atoms do not move; the others have
             // list slots.
             R pm1 = R(0), pm2 = R(0);   // this thread's two longest paths
-            if (!shift) {
+            if (!REED_RARE(shift)) {
 #pragma unroll 1
                 for (int k = tid; k < S->active_count; k += blockDim.x) {
                     const int i = W.slot_atom[k];
@@ -2620,7 +2637,7 @@ __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : t
                 m2 = fmax(fmin(m1, q1), fmax(m2, q2));
                 m1 = fmax(m1, q1);
             }
-            if (shift || m1 + m2 > H.skin) {
+            if (REED_RARE(shift || m1 + m2 > H.skin)) {
                 const int2 n = renew_lists<R, TT>(P, B, shift);
                 nbovf += n.x;
                 capovf += n.y;
@@ -2642,6 +2659,7 @@ __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : t
             }
             mark(PH_FORCE);
             if (lead && tid < 32) ion_step<R, false>(P, B, H, S, (int)blockDim.x >> 5, vt >> 5, tracing);
+            else if (lead && tid < 64) count_step<R>(S, (int)blockDim.x >> 5);
             team_sync();
             follow();
             const int ev = S->event;
