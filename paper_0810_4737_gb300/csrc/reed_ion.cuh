@@ -497,7 +497,7 @@ __device__ int acquire_track(const DevParams& P, const DevBuf& B, Head* S, IonWi
             S->pidx = (long long)k;
             S->src = ((long long)k < P.n_primaries) ? SRC_PRIMARY : SRC_NONE;
         }
-        if (S->src == SRC_NONE && B.pool) {
+        if (S->src == SRC_NONE && B.pool && P.nthr > 0) {   // (no clones without cloning depths)
             // out of work: take a donated clone, or stop once every CTA is
             // idle and no record is reserved or held
             bool idle = false;

@@ -2496,7 +2496,7 @@ __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : t
                 S->pidx = (long long)k;
                 S->src = ((long long)k < P.n_primaries) ? SRC_PRIMARY : SRC_NONE;
             }
-            if (S->src == SRC_NONE && B.pool) {
+            if (S->src == SRC_NONE && B.pool && P.nthr > 0) {   // (no clones without cloning depths)
                 // out of work: take a donated clone, or stop once every CTA is
                 // idle and no record is reserved or held
                 bool idle = false;

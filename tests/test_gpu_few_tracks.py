@@ -60,3 +60,13 @@ def test_damage_of_a_single_track_is_deposited_once(R):
     a, _, da = _records(R, w, 1, 0)
     b, _, db = _records(R, w, 1, 0, ctas_per_sm=1)
     assert a.tobytes() == b.tobytes() and np.allclose(da[0], db[0], rtol=1e-12, atol=0)
+
+
+def test_first_epoch_of_an_adaptive_run(R):
+    """Launched inside a captured graph, without cloning and with few tracks."""
+    w = workload("as10kev_si_300k_tersoff", energy=500.0, thresholds=[], step_cap=600)
+    ref, _, _ = _records(R, w, 20, 0)
+    w = workload("as10kev_si_300k_tersoff", energy=500.0, thresholds=[15.0, 30.0], step_cap=600)
+    rec, st, _ = _records(R, w, 50, 0, adaptive=True, n_initial=20, epoch_size=30, record_capacity=4000)
+    assert st["primaries"] == 50
+    assert rec[:20].tobytes() == ref.tobytes()
