@@ -755,9 +755,9 @@ int reed_run(reed_ctx* ctx, double ion_Z, double ion_M, double energy_eV, double
             if ((rc = dev_alloc(ctx, &ctx->d_pool, pool_need))) return rc;
             ctx->pool_bytes = pool_need;
         }
-        if (L.grid + 3 > ctx->pool_state_cap) {
-            if ((rc = dev_alloc(ctx, &ctx->d_pool_state, sizeof(unsigned) * (size_t)(L.grid + 3)))) return rc;
-            ctx->pool_state_cap = L.grid + 3;
+        if (L.grid + REED_POOL_CTL > ctx->pool_state_cap) {
+            if ((rc = dev_alloc(ctx, &ctx->d_pool_state, sizeof(unsigned) * (size_t)(L.grid + REED_POOL_CTL)))) return rc;
+            ctx->pool_state_cap = L.grid + REED_POOL_CTL;
         }
         B.pool = ctx->d_pool;
         B.pool_state = ctx->d_pool_state;
@@ -872,7 +872,7 @@ int reed_run(reed_ctx* ctx, double ion_Z, double ion_M, double energy_eV, double
                     cudaSuccess)
                 return e;
             if (B.pool &&
-                (e = cudaMemsetAsync(B.pool_state, 0, sizeof(unsigned) * (size_t)(B.pool_slots + 3), s)) != cudaSuccess)
+                (e = cudaMemsetAsync(B.pool_state, 0, sizeof(unsigned) * (size_t)(B.pool_slots + REED_POOL_CTL), s)) != cudaSuccess)
                 return e;
             if (o.adaptive && x.nthr > 0) {
                 double* hrow = ctx->d_thr_hist + (size_t)REED_MAX_THR * row++;

@@ -45,6 +45,7 @@ template <typename R> struct IonShared {
     IonState<R> ion;           // id, keys; complete only in records
     double thr[REED_MAX_THR];  // this track's cloning depths (frozen while it runs)
     int nthr, src, top, slot;
+    int was_busy;              // this CTA is counted among its SM's tracks
     int need_count, active_count, nhit0;   // build_ion_list: entries of the list, integrated atoms, hits
     long long pidx;
     unsigned long long cnt[ION_NCOUNT];
@@ -492,18 +493,36 @@ __device__ int acquire_track(const DevParams& P, const DevBuf& B, Head* S, IonWi
             S->src = SRC_CLONE;
         } else if (P.stop_after > 0 && (long long)(*(volatile unsigned long long*)B.finished) >= P.stop_after) {
             S->src = SRC_NONE;   // enough tracks collected: hand out no more primaries
+        } else if (B.pool && (long long)blockIdx.x >= P.n_primaries) {
+            S->src = SRC_NONE;   // the first CTAs, which are spread over the SMs, take one primary each
         } else {
             const unsigned long long k = atomicAdd(B.next, 1ull);
             S->pidx = (long long)k;
             S->src = ((long long)k < P.n_primaries) ? SRC_PRIMARY : SRC_NONE;
         }
+        // Tracks followed on each SM.  A clone is best taken where few others
+        // share the SM, so an idle CTA lets a record lie for one poll per track
+        // on its SM; a CTA of an idle SM takes it at once.
+        unsigned smid;
+        asm("mov.u32 %0, %%smid;" : "=r"(smid));
+        unsigned* busy = B.pool ? &B.pool_ctl[3 + smid % REED_POOL_SMS] : nullptr;
+        if (B.pool && S->was_busy != (S->src != SRC_NONE)) {
+            if (S->src != SRC_NONE) atomicAdd(busy, 1u);
+            else atomicSub(busy, 1u);
+            S->was_busy = S->src != SRC_NONE;
+        }
         if (S->src == SRC_NONE && B.pool && P.nthr > 0) {   // (no clones without cloning depths)
+            unsigned seen = 0;
             // out of work: take a donated clone, or stop once every CTA is
             // idle and no record is reserved or held
             bool idle = false;
             for (long long it = 0;; ++it) {
-                const int sl = *(volatile unsigned*)&B.pool_ctl[2] > 0u ? pool_claim(B, POOL_FULL, POOL_READING) : -1;
+                seen = *(volatile unsigned*)&B.pool_ctl[2] > 0u ? seen + 1u : 0u;
+                const int sl =
+                    seen && seen > *(volatile unsigned*)busy ? pool_claim(B, POOL_FULL, POOL_READING) : -1;
                 if (sl >= 0) {
+                    atomicAdd(busy, 1u);
+                    S->was_busy = 1;
                     atomicSub(&B.pool_ctl[2], 1u);
                     if (idle) atomicSub(&B.pool_ctl[0], 1u);
                     S->slot = sl;
@@ -807,6 +826,7 @@ __global__ void __launch_bounds__(ADJ ? 256 : 32, (ADJ ? (sizeof(R) == 4 ? 2 : 1
     long long t_mark = clock64();
     if (tid == 0) {
         S->top = 0;
+        S->was_busy = 0;
         for (int c = 0; c < ION_NCOUNT; ++c) S->cnt[c] = 0;
     }
     if (ADJ) __syncthreads();

@@ -78,6 +78,7 @@ template <typename R> struct TrackShared {
     unsigned mark[6];     // clocks: the end of the last step's forces, then of each phase of this step
     long long moved_from, centred_from, steps_from;   // see count_listed; steps before this CTA took the track
     int status, top, nclone, slot;
+    int was_busy;         // (see IonShared; the adjoint has no pool)
     int need_count, active_count;
     int nhit0;            // ion-target-only model: atoms within the cutoff at the last list build
     unsigned long long cnt[REED_NCOUNT];  // counters of this CTA (C_*; ion-target-only model: ION_*), flushed at exit
