@@ -158,7 +158,7 @@ struct DevBuf {
     // that busy CTAs donate while some CTA is idle
     unsigned char* pool;            // pool_slots x entry_bytes
     unsigned* pool_state;           // per slot: POOL_EMPTY / WRITING / FULL / READING
-    unsigned* pool_ctl;             // [0] idle CTAs, [1] records reserved or held, [2] records published
+    unsigned* pool_ctl;             // [0] idle CTAs, [1] records reserved or held, [2] records published, [3..] tracks per SM
     int pool_slots;
     double* wsum;                   // W_*
     unsigned long long* next;       // primary queue head

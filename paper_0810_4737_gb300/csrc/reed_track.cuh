@@ -2034,7 +2034,9 @@ __device__ __noinline__ void trace_step(const DevParams& P, const DevBuf& B, con
 // The rest of the CTA waits here, so what counts is the length of the chain.
 // Lanes 0-2 hold one component each and lane 3 the time: an FP64 addition
 // (some hundred cycles for the SM's FP64 unit) is issued twice a step and not
-// six times, and a column of the partial sums is added by one lane each.
+// six times, a column of the partial sums is added by one lane each, and the
+// counters are the second warp's: 7.9k -> 2.9k cycles of an As step's 29k (one
+// thread with rolled loops: 4.0k).
 // `rows` warps left partial sums; those of the ion (columns 0-3) are in `vrows`
 // rows.
 template <typename R, bool BEGIN>
@@ -2423,7 +2425,8 @@ template <typename R, int TT> inline int track_threads(int act_cap)
 // + 35 KB, ion 9 KB, lists) goes through the instruction cache once per step,
 // and a warp that runs alone waits for each line of it.  So the rare parts are
 // calls (REED_WINDOW), short loops are not unrolled, and the groups of 8 and 16
-// lanes share their code: 4096 As ions of 10 keV 1139 -> 977 ms.
+// lanes share their code: 4096 As ions of 10 keV 1139 -> 977 ms, and 823 ms with
+// the counters out of the ion update (see ion_step).
 template <typename R, int TT, int MAX_THREADS = track_max_threads<R, TT>(), bool TEAM = false>
 __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : track_min_ctas<R, TT>()))
     reed_track_kernel(const __grid_constant__ DevParams P, const __grid_constant__ DevBuf B, const int vt)
