@@ -245,9 +245,10 @@ double lindhard_gamma_unit(const reed_ctx* ctx, double Z1, double M1)
     return g * std::sqrt(M1 / 2.0);
 }
 
-// Rows of Tersoff bond storage: atoms of a perfect bulk window that are
-// integrated or within the list radius of an integrated atom, plus 25 %
+// Rows of Tersoff bond storage at least: atoms of a perfect bulk window that
+// are integrated or within the list radius of an integrated atom, plus 25 %
 // head-room for disorder and cascades (capped at the window size).
+// list_capacity adds what the shared memory leaves.
 int bond_capacity(const DevParams& P, double skin)
 {
     if (P.tt == REED_TT_NONE) return 0;
@@ -378,6 +379,57 @@ int make_params(reed_ctx* ctx, DevParams& P, double Z1, double M1, double E, dou
         const int k = P.n - 2 * P.margin;
         P.act_cap = k * k * k * P.nb;
     }
+    return REED_OK;
+}
+
+// REED_E_NEIGHBOR, with the counters (since the last reset) that say why.
+int neighbor_error(reed_ctx* ctx, const unsigned long long* c)
+{
+    return fail(ctx, REED_E_NEIGHBOR,
+                "neighbour lists did not fit and forces were incomplete: %llu entries found no room in their row or an "
+                "overflow row (nb_overflow), %llu atoms no row in the list table (bond_cap_overflow)",
+                c[C_NBOVF], c[C_CAPOVF]);
+}
+
+// The launch shape of a run: shared memory, tracks per SM and the rows of the
+// list table.  Integrated atoms that a cascade throws into the frozen layer
+// make more frozen atoms needed than bond_capacity counts on: of 446 000 As
+// tracks of 10 keV two ran out of the 456 rows of a 5^3-cell window, by 2 and 4.
+// So the table takes the shared memory that as many tracks per SM leave unused,
+// up to a row for every atom of the window (the mixed form: some 550 rows).  Refreshes still give way to a build where they
+// did, at refresh_cap: the order of the lists, and with it every rounding, does
+// not depend on the size of the table.
+int list_capacity(reed_ctx* ctx, DevParams& P, bool f64, size_t optin, int device, LaunchCfg& L, int* occ)
+{
+    const int tt = P.tt, base = P.bond_cap;
+    auto bytes = [&](int cap) {
+        return f64 ? reed_f64::track_smem_bytes(tt, P.na, cap, P.adjoint, P.g_nbins, P.act_cap)
+                   : reed_f32::track_smem_bytes(tt, P.na, cap, P.adjoint, P.g_nbins, P.act_cap);
+    };
+    auto fit = [&](int cap) {   // tracks per SM with `cap` rows
+        P.bond_cap = cap;
+        L.smem = bytes(cap);
+        return f64 ? reed_f64::occupancy(tt, L.threads, L.smem, occ, P.adjoint, P.act_cap)
+                   : reed_f32::occupancy(tt, L.threads, L.smem, occ, P.adjoint, P.act_cap);
+    };
+    P.refresh_cap = base;
+    if (bytes(base) > optin)
+        return fail(ctx, REED_E_SMEM, "window of %d atoms needs %zu B of shared memory (max %zu)", P.na, bytes(base), optin);
+    CK(fit(base));
+    const int tracks = *occ;
+    if (tt != REED_TT_TERSOFF || base >= P.na || tracks < 1) return REED_OK;
+    int sm = 0, reserved = 0;
+    CK(cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device));
+    CK(cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, device));
+    const size_t room = std::min(optin, (size_t)std::max(sm / tracks - reserved, 0) / 1024 * 1024);
+    int lo = base, hi = P.na;   // the most rows that fit
+    while (lo < hi) {
+        const int m = (lo + hi + 1) / 2;
+        if (bytes(m) <= room) lo = m;
+        else hi = m - 1;
+    }
+    CK(fit(lo));
+    if (*occ != tracks) CK(fit(base));
     return REED_OK;
 }
 
@@ -717,21 +769,14 @@ int reed_run(reed_ctx* ctx, double ion_Z, double ion_M, double energy_eV, double
         P.adj_every = every;
         P.adj_nck = seg / every + 1;
     }
-    const size_t smem = f64 ? reed_f64::track_smem_bytes(tt, P.na, P.bond_cap, P.adjoint, P.g_nbins, P.act_cap)
-                            : reed_f32::track_smem_bytes(tt, P.na, P.bond_cap, P.adjoint, P.g_nbins, P.act_cap);
-    if (smem > ctx->smem_optin)
-        return fail(ctx, REED_E_SMEM, "window of %d atoms needs %zu B of shared memory (max %zu)", P.na, smem,
-                    ctx->smem_optin);
     LaunchCfg L;
     const int pi = f64 ? 1 : 0, ai = P.adjoint ? 1 : 0;
     const bool tuned = !o.threads_per_track && !o.ctas_per_sm && ctx->tuned_threads[pi][ai] > 0;
     L.threads = o.threads_per_track ? o.threads_per_track
                                     : (tuned ? ctx->tuned_threads[pi][ai] : (tt == REED_TT_NONE ? 64 : 256));
-    L.smem = smem;
     int occ = 0;
-    CK(f64 ? reed_f64::occupancy(tt, L.threads, smem, &occ, P.adjoint, P.act_cap)
-           : reed_f32::occupancy(tt, L.threads, smem, &occ, P.adjoint, P.act_cap));
-    if (occ < 1) return fail(ctx, REED_E_SMEM, "kernel does not fit on an SM (%zu B shared, %d threads)", smem, L.threads);
+    if ((rc = list_capacity(ctx, P, f64, ctx->smem_optin, ctx->device, L, &occ))) return rc;
+    if (occ < 1) return fail(ctx, REED_E_SMEM, "kernel does not fit on an SM (%zu B shared, %d threads)", L.smem, L.threads);
     L.ctas_per_sm = o.ctas_per_sm ? std::min(o.ctas_per_sm, occ) : (tuned ? std::min(ctx->tuned_ctas[pi][ai], occ) : occ);
     L.grid = ctx->sms * L.ctas_per_sm;
     L.sms = ctx->sms;
@@ -926,10 +971,11 @@ int reed_run(reed_ctx* ctx, double ion_Z, double ion_M, double energy_eV, double
         return fail(ctx, REED_E_TIMEOUT, "an idle CTA stopped waiting for the shared clone pool: tracks may be missing");
     if (status & ERR_NONFINITE) return fail(ctx, REED_E_NONFINITE, "a track became non-finite (see reed_stats)");
     if (status & ERR_QUEUE) return fail(ctx, REED_E_QUEUE_FULL, "clone stack overflow: clones dropped");
-    if (status & ERR_NEIGHBOR)
-        return fail(ctx, REED_E_NEIGHBOR,
-                    "a neighbour list outgrew its overflow row or the overflow rows ran out (see nb_overflow, "
-                    "bond_cap_overflow in reed_stats): forces were incomplete");
+    if (status & ERR_NEIGHBOR) {
+        unsigned long long c[REED_NCOUNT];
+        CK(cudaMemcpy(c, ctx->d_counters, sizeof(c), cudaMemcpyDeviceToHost));
+        return neighbor_error(ctx, c);
+    }
     return REED_OK;
 }
 
@@ -1594,16 +1640,11 @@ extern "C" int reed_run_static(const reed_lattice* lat, const reed_species* sp, 
 
     const int tt = P.tt;
     const bool f64 = o.precision == REED_PREC_FP64;
-    const size_t smem = f64 ? reed_f64::track_smem_bytes(tt, P.na, P.bond_cap, 0, P.g_nbins, P.act_cap)
-                            : reed_f32::track_smem_bytes(tt, P.na, P.bond_cap, 0, P.g_nbins, P.act_cap);
-    if (smem > (size_t)optin)
-        return fail(nullptr, REED_E_SMEM, "window of %d atoms needs %zu B of shared memory (max %d)", P.na, smem, optin);
     LaunchCfg L;
     L.threads = o.threads_per_track ? o.threads_per_track : (tt == REED_TT_NONE ? 64 : 256);
-    L.smem = smem;
     int occ = 0;
-    CK(f64 ? reed_f64::occupancy(tt, L.threads, smem, &occ, P.adjoint, P.act_cap)
-           : reed_f32::occupancy(tt, L.threads, smem, &occ, P.adjoint, P.act_cap));
+    int rc = list_capacity(nullptr, P, f64, (size_t)optin, desc.device, L, &occ);
+    if (rc) return rc;
     if (occ < 1) return fail(nullptr, REED_E_SMEM, "kernel does not fit on an SM");
     L.ctas_per_sm = o.ctas_per_sm ? std::min(o.ctas_per_sm, occ) : occ;
 
@@ -1627,8 +1668,7 @@ extern "C" int reed_run_static(const reed_lattice* lat, const reed_species* sp, 
     L.sms = desc.sms;
 
     unsigned char* base = nullptr;
-    int rc = static_scratch((void**)&base);
-    if (rc) return rc;
+    if ((rc = static_scratch((void**)&base))) return rc;
     B.counters = reinterpret_cast<unsigned long long*>(base);
     B.wsum = reinterpret_cast<double*>(base + 256);
     B.next = reinterpret_cast<unsigned long long*>(base + 512);
@@ -1696,9 +1736,6 @@ extern "C" int reed_run_static(const reed_lattice* lat, const reed_species* sp, 
     }
     if (status & ERR_NONFINITE) return fail(nullptr, REED_E_NONFINITE, "a track became non-finite");
     if (status & ERR_QUEUE) return fail(nullptr, REED_E_QUEUE_FULL, "clone stack overflow: clones dropped");
-    if (status & ERR_NEIGHBOR)
-        return fail(nullptr, REED_E_NEIGHBOR,
-                    "a neighbour list outgrew its overflow row or the overflow rows ran out (see nb_overflow): "
-                    "forces were incomplete");
+    if (status & ERR_NEIGHBOR) return neighbor_error(nullptr, c);
     return REED_OK;
 }

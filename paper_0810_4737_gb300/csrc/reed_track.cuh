@@ -1139,7 +1139,7 @@ __device__ bool refresh_lists(const DevParams& P, const HotParams<R>& H, Win<R, 
     for (int i = i0; i < i1; ++i) np += W.need_map[i] == REED_PENDING;
     int op, dummy, tp, dummy_t;
     block_scan2<R>(S, np, 0, op, dummy, tp, dummy_t);
-    if (nneed0 + tp > P.bond_cap) {
+    if (nneed0 + tp > P.refresh_cap) {
         __syncthreads();
         return false;
     }
