@@ -865,7 +865,9 @@ __global__ void __launch_bounds__(ADJ ? 256 : 32, (ADJ ? (sizeof(R) == 4 ? 2 : 1
             }
         }
         if (ADJ) __syncthreads();
-        if (S->src == SRC_NONE) break;
+        const int src = S->src;
+        if (!ADJ) __syncwarp();   // (lane 0 goes on to write the next track's; an adjoint run ends on a barrier)
+        if (src == SRC_NONE) break;
         if constexpr (ADJ) {
             // truncated-segment sensitivities of the final depth
             if (adjbase && B.grads && S->rec_index >= 0) {
