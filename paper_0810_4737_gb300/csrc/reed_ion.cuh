@@ -282,9 +282,11 @@ __device__ __noinline__ R build_ion_list(const DevParams& P, const DevBuf& B, He
                 const R r2 = dist2(dx, dy, dz);
                 const bool moving = act && (v.x != R(0) || v.y != R(0) || v.z != R(0));
                 in_range = r2 < H.rc2;
-                in_list = in_range || r2 < rl2 || moving || t.x != R(0);
+                // (an atom whose force underflows can still have a density weight)
+                const bool term_on = t.x != R(0) || v.w != R(0);
+                in_list = in_range || r2 < rl2 || moving || term_on;
                 if (!in_range) {
-                    if (clear && t.x != R(0)) {
+                    if (clear && term_on) {
                         term[i] = none;
                         vel[i].w = R(0);
                     }
@@ -336,7 +338,7 @@ __device__ __forceinline__ bool ion_move_atom(const HotParams<R>& H, IonWin<R>& 
     const R r2 = dist2(dx, dy, dz);
     const bool in = r2 < H.rc2;
     if (!in) {
-        if (t.x != R(0)) {   // it has just left the cutoff
+        if (t.x != R(0) || v.w != R(0)) {   // it has just left the cutoff
             W.term[i] = {R(0), R(0), R(0), R(0)};
             v.w = R(0);
         }

@@ -43,3 +43,22 @@ def test_windows_and_summation_widths(R, O, name, n, margin, threads, prec):
         assert k == STEPS
         np.testing.assert_allclose(traj[t, :, :3], ref[:, :3], rtol=0, atol=1e-9 if prec else 1e-4)
         assert np.array_equal(anchors[t], ref_anchors)
+
+
+def test_density_of_atoms_without_a_force(R, O):
+    """A correction exp(c) that underflows in FP32 leaves the pair terms zero and
+    the local density as it is: atoms that the ion has left behind must not stay
+    in it.  (Long density range and a steep taper, so that an atom's weight is
+    still large when it leaves the cutoff.)  The drag on a straight flight through
+    20 A: velocities to 1e-5, some hundred FP32 roundings; the drag changes them
+    by more than 1e-2."""
+    w = workload("b1kev_si_0k_zbl", sigma=0.076, spline_c=[-2000.0] * 6, s_loc=1.0, lam_loc=5.0, rt=4.9, s_e=20.0)
+    p = O.params(w)
+    steps = 400
+    with R.Reed(w) as ctx:
+        ctx.run(n_ions=2, seed=11, trace_tracks=2, trace_steps=steps, step_cap=steps)
+        traj, _ = ctx.trace(2, steps)
+    for t in range(2):
+        ref, _ = O.trace(p, 11, t, steps)
+        assert abs(ref[-1, 6] / ref[0, 6] - 1) > 1e-2
+        np.testing.assert_allclose(traj[t, :, 4:7], ref[:, 4:7], rtol=1e-5, atol=0)
