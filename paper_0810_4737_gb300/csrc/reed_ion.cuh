@@ -183,7 +183,7 @@ __device__ __forceinline__ bool regs_prologue(const DevParams& P, const HotParam
     R dt = H.dt_max;
     if (vmax * dt > H.dx_max) dt = H.dx_max / vmax;
     if (H.de_max > R(0)) {
-        const R pw = max(fabs(I.f[0] * I.v[0] + I.f[1] * I.v[1] + I.f[2] * I.v[2]), I.pmax);
+        const R pw = max(fabs(dot3(I.f[0], I.f[1], I.f[2], I.v[0], I.v[1], I.v[2])), I.pmax);
         if (pw * dt > H.de_max) {
             dt = H.de_max / pw;
             if (vmax * dt < H.dx_min) dt = H.dx_min / vmax;
@@ -373,7 +373,7 @@ __device__ __forceinline__ void ion_pair_pass(const DevParams& P, const HotParam
             v.y = fma(kk, fy, v.y);
             v.z = fma(kk, fz, v.z);
             vm = max(vm, dist2(v.x, v.y, v.z));
-            if (H.de_max > R(0)) pm = max(pm, fabs(fx * v.x + fy * v.y + fz * v.z));
+            if (H.de_max > R(0)) pm = max(pm, fabs(dot3(fx, fy, fz, v.x, v.y, v.z)));
         }
         W.vel[i] = v;
     }

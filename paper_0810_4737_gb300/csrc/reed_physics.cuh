@@ -18,6 +18,11 @@ __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, 
 __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
 // x^2 + y^2 + z^2
 template <typename R> __device__ __forceinline__ R dist2(R x, R y, R z) { return fma(z, z, fma(x, x, mul_rn(y, y))); }
+// ax bx + ay by + az bz
+template <typename R> __device__ __forceinline__ R dot3(R ax, R ay, R az, R bx, R by, R bz)
+{
+    return fma(az, bz, fma(ax, bx, mul_rn(ay, by)));
+}
 
 // ZBL universal screening (Sec. 2 "First"; Ziegler, Biersack, Littmark 1985):
 // phi(x) = sum_i c_i exp(-d_i x) with x = r / a_U,

@@ -1973,8 +1973,10 @@ template <typename R> __device__ void launch_primary(const DevParams& P, IonStat
 template <typename R> __device__ void set_frame(const DevParams& P, TrackShared<R>* S)
 {
     const IonState<R>& I = S->ion;
-    for (int d = 0; d < 3; ++d) S->rel[d] = R(I.x[d] - (double)I.A[d] * P.a);
-    const double z0 = (double)I.A[2] * P.a;
+    // (in these roundings in every kernel, see regs_frame)
+    const double z0 = __dmul_rn((double)I.A[2], P.a);
+    for (int d = 0; d < 2; ++d) S->rel[d] = R(fma(-(double)I.A[d], P.a, I.x[d]));
+    S->rel[2] = R(__dsub_rn(I.x[2], z0));
     if (P.bulk) {   // no surface; the depth checks run on the distance from the start
         S->zthr = I.level < S->nthr ? R(-1e30) : R(1e30);
         S->zback = R(-1e30);
@@ -2118,7 +2120,7 @@ __device__ __forceinline__ int ion_step(const DevParams& P, const DevBuf& B, con
         if (vmax * dt > H.dx_max) dt = H.dx_max / vmax;
         if (H.de_max > R(0)) {   // energy term: |dE_kin| <= de_max per step for every particle
             const R f0 = __shfl_sync(FULL, f, 0), f1 = __shfl_sync(FULL, f, 1), f2 = __shfl_sync(FULL, f, 2);
-            const R pw = max(fabs(f0 * v0 + f1 * v1 + f2 * v2), pmax);
+            const R pw = max(fabs(dot3(f0, f1, f2, v0, v1, v2)), pmax);
             if (pw * dt > H.de_max) {
                 dt = H.de_max / pw;
                 if (vmax * dt < H.dx_min) dt = H.dx_min / vmax;   // a step that moves nothing stalls
