@@ -248,7 +248,7 @@ double lindhard_gamma_unit(const reed_ctx* ctx, double Z1, double M1)
 // Rows of Tersoff bond storage at least: atoms of a perfect bulk window that
 // are integrated or within the list radius of an integrated atom, plus 25 %
 // head-room for disorder and cascades (capped at the window size).
-// list_capacity adds what the shared memory leaves.
+// launch_shape adds what the shared memory leaves.
 int bond_capacity(const DevParams& P, double skin)
 {
     if (P.tt == REED_TT_NONE) return 0;
@@ -391,31 +391,62 @@ int neighbor_error(reed_ctx* ctx, const unsigned long long* c)
                 c[C_NBOVF], c[C_CAPOVF]);
 }
 
+// Whether a block of `threads` threads follows a track of the ion-target-only
+// model (mixed form), and not one warp; warps, blocks: how many tracks an SM
+// holds either way.  A block takes a step sooner and more of an SM: it is taken
+// where a width of 128 or 256 is asked for and warps would be idle, with two
+// tracks per SM or fewer, or in a window so large that an SM's shared memory
+// holds three tracks or fewer (at a width of 128 only if it holds more blocks:
+// their windows need no list).  Measured, one warp -> block, 1200 steps: width
+// 256, 300 tracks: B in 3^3 cells of Si 3.24 -> 2.30 ms, U in 3^3 of UO2 3.99 ->
+// 2.78; 2400 tracks, U in 5^3 49.7 -> 26.1, in 6^3 129.6 -> 81.3.  Width 128, 300
+// tracks: 2.81 -> 2.60 and 3.56 -> 3.03; 2400 U in 5^3 (2 warps, 3 blocks) 46.2 ->
+// 34.9.  On the other side of the line, width 256: 600 B in 3^3 3.26 -> 4.52, 2400
+// U in 4^3 18.8 -> 19.3; width 128: 2400 B in 6^3 (2 and 2) 46.9 -> 49.0; width 64:
+// 300 B in 3^3 2.58 -> 3.38.  The FP64 form is bound by its pipe, and one warp is
+// the faster one from 3^3 cells on (300 B, width 256: 3.53 -> 4.48).
+bool ion_by_block(const DevParams& P, int threads, int sms, int warps, int blocks)
+{
+    if (warps <= 3) return threads == 256 || blocks > warps;
+    return P.nthr == 0 && P.n_primaries <= 2 * (int64_t)sms;
+}
+
 // The launch shape of a run: shared memory, tracks per SM and the rows of the
 // list table.  Integrated atoms that a cascade throws into the frozen layer
 // make more frozen atoms needed than bond_capacity counts on: of 446 000 As
 // tracks of 10 keV two ran out of the 456 rows of a 5^3-cell window, by 2 and 4.
 // So the table takes the shared memory that as many tracks per SM leave unused,
-// up to a row for every atom of the window (the mixed form: some 550 rows).  Refreshes still give way to a build where they
-// did, at refresh_cap: the order of the lists, and with it every rounding, does
-// not depend on the size of the table.
-int list_capacity(reed_ctx* ctx, DevParams& P, bool f64, size_t optin, int device, LaunchCfg& L, int* occ)
+// up to a row for every atom of the window (the mixed form: some 550 rows).
+// Refreshes still give way to a build where they did, at refresh_cap: the order
+// of the lists, and with it every rounding, does not depend on the size of the
+// table.
+int launch_shape(reed_ctx* ctx, DevParams& P, bool f64, size_t optin, int device, LaunchCfg& L, int* occ)
 {
     const int tt = P.tt, base = P.bond_cap;
     auto bytes = [&](int cap) {
-        return f64 ? reed_f64::track_smem_bytes(tt, P.na, cap, P.adjoint, P.g_nbins, P.act_cap)
-                   : reed_f32::track_smem_bytes(tt, P.na, cap, P.adjoint, P.g_nbins, P.act_cap);
+        return f64 ? reed_f64::track_smem_bytes(tt, P.na, cap, P.adjoint, P.g_nbins, P.act_cap, L.block)
+                   : reed_f32::track_smem_bytes(tt, P.na, cap, P.adjoint, P.g_nbins, P.act_cap, L.block);
     };
     auto fit = [&](int cap) {   // tracks per SM with `cap` rows
         P.bond_cap = cap;
         L.smem = bytes(cap);
-        return f64 ? reed_f64::occupancy(tt, L.threads, L.smem, occ, P.adjoint, P.act_cap)
-                   : reed_f32::occupancy(tt, L.threads, L.smem, occ, P.adjoint, P.act_cap);
+        return f64 ? reed_f64::occupancy(tt, L.threads, L.smem, occ, P.adjoint, P.act_cap, L.block)
+                   : reed_f32::occupancy(tt, L.threads, L.smem, occ, P.adjoint, P.act_cap, L.block);
     };
     P.refresh_cap = base;
+    L.block = false;
     if (bytes(base) > optin)
         return fail(ctx, REED_E_SMEM, "window of %d atoms needs %zu B of shared memory (max %zu)", P.na, bytes(base), optin);
     CK(fit(base));
+    if (tt == REED_TT_NONE && !P.adjoint && !f64 && (L.threads == 128 || L.threads == 256)) {
+        const int warps = *occ;
+        L.block = true;
+        CK(fit(base));
+        if (*occ >= 1 && ion_by_block(P, L.threads, L.sms, warps, *occ)) return REED_OK;
+        L.block = false;
+        CK(fit(base));
+        return REED_OK;
+    }
     const int tracks = *occ;
     if (tt != REED_TT_TERSOFF || base >= P.na || tracks < 1) return REED_OK;
     int sm = 0, reserved = 0;
@@ -774,12 +805,12 @@ int reed_run(reed_ctx* ctx, double ion_Z, double ion_M, double energy_eV, double
     const bool tuned = !o.threads_per_track && !o.ctas_per_sm && ctx->tuned_threads[pi][ai] > 0;
     L.threads = o.threads_per_track ? o.threads_per_track
                                     : (tuned ? ctx->tuned_threads[pi][ai] : (tt == REED_TT_NONE ? 64 : 256));
+    L.sms = ctx->sms;
     int occ = 0;
-    if ((rc = list_capacity(ctx, P, f64, ctx->smem_optin, ctx->device, L, &occ))) return rc;
+    if ((rc = launch_shape(ctx, P, f64, ctx->smem_optin, ctx->device, L, &occ))) return rc;
     if (occ < 1) return fail(ctx, REED_E_SMEM, "kernel does not fit on an SM (%zu B shared, %d threads)", L.smem, L.threads);
     L.ctas_per_sm = o.ctas_per_sm ? std::min(o.ctas_per_sm, occ) : (tuned ? std::min(ctx->tuned_ctas[pi][ai], occ) : occ);
     L.grid = ctx->sms * L.ctas_per_sm;
-    L.sms = ctx->sms;
 
     // clone stacks: one record per cloning level per CTA
     DevBuf B;
@@ -1642,8 +1673,9 @@ extern "C" int reed_run_static(const reed_lattice* lat, const reed_species* sp, 
     const bool f64 = o.precision == REED_PREC_FP64;
     LaunchCfg L;
     L.threads = o.threads_per_track ? o.threads_per_track : (tt == REED_TT_NONE ? 64 : 256);
+    L.sms = desc.sms;
     int occ = 0;
-    int rc = list_capacity(nullptr, P, f64, (size_t)optin, desc.device, L, &occ);
+    int rc = launch_shape(nullptr, P, f64, (size_t)optin, desc.device, L, &occ);
     if (rc) return rc;
     if (occ < 1) return fail(nullptr, REED_E_SMEM, "kernel does not fit on an SM");
     L.ctas_per_sm = o.ctas_per_sm ? std::min(o.ctas_per_sm, occ) : occ;
@@ -1665,7 +1697,6 @@ extern "C" int reed_run_static(const reed_lattice* lat, const reed_species* sp, 
                     "than the %zu B static scratch",
                     per_cta * (size_t)desc.sms, desc.sms, P.nthr, B.entry_bytes, B.spill_stride, room);
     L.grid = desc.sms * L.ctas_per_sm;
-    L.sms = desc.sms;
 
     unsigned char* base = nullptr;
     if ((rc = static_scratch((void**)&base))) return rc;

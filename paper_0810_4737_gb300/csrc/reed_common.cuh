@@ -115,7 +115,7 @@ struct DevParams {
     double b_rt, b_rc, b_lo, b_hi;
     double b_zk[3], b_zia[3];
     int bond_cap;                      // neighbour-list rows (Tersoff: needed atoms)
-    int refresh_cap;                   // rows past which a list refresh gives way to a build (see list_capacity)
+    int refresh_cap;                   // rows past which a list refresh gives way to a build (see launch_shape)
     int nl_check;                      // compare every list with a brute-force search after each build
     int act_cap;                       // integrated atoms a window can hold (rows of the per-bond forces)
     // electronic stopping (Sec. 2 "Third")

@@ -2262,21 +2262,86 @@ __device__ __forceinline__ void copy_window(const DevParams& P, Win<R, TT>& W, u
     }
 }
 
+// A step of the ion-target-only model by a block of threads (see
+// ion_by_block): first half kick and drift, window move, pair term with the ion
+// and second half kick of each atom in one pass, its state in registers; with
+// START the forces at the start of a track only.  In the roundings of the
+// one-warp kernel (reed_ion.cuh), so that a track's bits are the same.  Returns
+// the integrated atoms of this thread.
+template <typename R, bool START>
+__device__ __forceinline__ unsigned ion_block_pass(const DevParams& P, const DevBuf& B, const HotParams<R>& H,
+                                                   Win<R, REED_TT_NONE>& W, R dt, R hdt, bool shift, Partial<R>& q)
+{
+    TrackShared<R>* S = W.S;
+    const R ix = S->rel[0], iy = S->rel[1], iz = S->rel[2];
+    unsigned moved = 0;
+    for (int i = threadIdx.x; i < P.na; i += blockDim.x) {
+        V4<R> p = W.pos[i], v = W.vel[i], f = W.frc[i];
+        if (!START && is_active(p)) {
+            ++moved;
+            const R k = hdt * of_species(H.invM2, p);
+            v.x = fma(k, f.x, v.x);
+            v.y = fma(k, f.y, v.y);
+            v.z = fma(k, f.z, v.z);
+            p.x = fma(dt, v.x, p.x);
+            p.y = fma(dt, v.y, p.y);
+            p.z = fma(dt, v.z, p.z);
+        }
+        if (!START && shift) {
+            const V4<R> p0 = p, v0 = v;
+            if (reanchor_atom<R>(P, H, S->ion.key, i, S->Aold, S->ion.A, p, v, f))
+                deposit_damage<R>(P, B, p0, v0, S->Aold, ldexp(1.0, -S->ion.level));
+        }
+        if (is_present(p)) {
+            const R dx = p.x - ix, dy = p.y - iy, dz = p.z - iz;
+            const R r2 = dist2(dx, dy, dz);
+            f = {R(0), R(0), R(0), R(0)};
+            if (r2 < H.rc2) {
+                R U, rw;
+                const R g = ion_pair<R>(H, P.spline_on, P.rho_on, is_second(p), r2, U, rw);
+                f.x = -mul_rn(g, dx);
+                f.y = -mul_rn(g, dy);
+                f.z = -mul_rn(g, dz);
+                q.fx = fma(g, dx, q.fx);
+                q.fy = fma(g, dy, q.fy);
+                q.fz = fma(g, dz, q.fz);
+                q.rho += rw;
+                q.pairs += 1;
+            }
+            if (!START && is_active(p)) {
+                const R kk = hdt * of_species(H.invM2, p);
+                v.x = fma(kk, f.x, v.x);
+                v.y = fma(kk, f.y, v.y);
+                v.z = fma(kk, f.z, v.z);
+                q.vmax2 = max(q.vmax2, dist2(v.x, v.y, v.z));
+                if (H.de_max > R(0)) q.pmax = max(q.pmax, fabs(dot3(f.x, f.y, f.z, v.x, v.y, v.z)));
+            }
+        }
+        W.pos[i] = p;
+        W.vel[i] = v;
+        W.frc[i] = f;
+    }
+    return moved;
+}
+
 // Forces + (optionally) target bookkeeping at the start of a track.
 template <typename R, int TT>
-__device__ void initial_forces(const DevParams& P, const HotParams<R>& H, Win<R, TT>& W, int& nbovf, int& capovf,
-                               unsigned& triplets, int vt)
+__device__ void initial_forces(const DevParams& P, const DevBuf& B, const HotParams<R>& H, Win<R, TT>& W, int& nbovf,
+                               int& capovf, unsigned& triplets, int vt)
 {
-    build_neighbours<R, TT>(P, H, W, nbovf, capovf);
-    if (threadIdx.x == 0) ++W.S->cnt[C_REBUILDS];
-    __syncthreads();
+    if constexpr (TT != REED_TT_NONE) {
+        build_neighbours<R, TT>(P, H, W, nbovf, capovf);
+        if (threadIdx.x == 0) ++W.S->cnt[C_REBUILDS];
+        __syncthreads();
+    }
     if (P.nl_check) check_lists<R, TT>(P, H, W, H.rlist2);
     if constexpr (TT == REED_TT_TERSOFF) {
         ters_centres<R, TT>(H, W, triplets);
         __syncthreads();
     }
     Partial<R> q = {R(0), R(0), R(0), R(0), R(0), R(0), 0, 0};
-    force_phase<R, TT, false>(P, H, W, R(0), q, false);
+    if constexpr (TT == REED_TT_NONE) ion_block_pass<R, true>(P, B, H, W, R(0), R(0), false, q);
+    else force_phase<R, TT, false>(P, H, W, R(0), q, false);
     reduce_partials<R, TT>(W, q);
     __syncthreads();
     if (vt != (int)blockDim.x) {
@@ -2380,8 +2445,8 @@ __device__ __noinline__ int3 start_track(const DevParams& P, const DevBuf& B, bo
     int nbovf = 0, capovf = 0;
     unsigned triplets = 0;
     if (forces) {
-        initial_forces<R, TT>(P, H, W, nbovf, capovf, triplets, vt);
-    } else {
+        initial_forces<R, TT>(P, B, H, W, nbovf, capovf, triplets, vt);
+    } else if constexpr (TT != REED_TT_NONE) {
         build_neighbours<R, TT>(P, H, W, nbovf, capovf);
         if (threadIdx.x == 0) ++W.S->cnt[C_REBUILDS];
         __syncthreads();
@@ -2390,12 +2455,17 @@ __device__ __noinline__ int3 start_track(const DevParams& P, const DevBuf& B, bo
 }
 
 // ---------------------------------------------------------------------------
-// The persistent kernel of the models with target-target forces (the
-// ion-target-only model and its adjoint: reed_ion.cuh).
+// The persistent kernel of the models with target-target forces, and of the
+// ion-target-only model where a block of threads follows a track (ion_by_block;
+// one warp per track and the adjoint: reed_ion.cuh).
 // The second launch bound is the number of CTAs per SM the shared memory of
 // the workloads allows, so registers are budgeted for that occupancy.
 // ---------------------------------------------------------------------------
-template <typename R, int TT> constexpr int track_min_ctas() { return TT == REED_TT_TERSOFF && sizeof(R) == 4 ? 2 : 1; }
+template <typename R, int TT> constexpr int track_min_ctas()
+{
+    if (TT == REED_TT_NONE) return sizeof(R) == 4 ? 3 : 2;
+    return TT == REED_TT_TERSOFF && sizeof(R) == 4 ? 2 : 1;
+}
 
 
 // Threads of a track's CTA at most.  The pair-list model: one track fills an
@@ -2433,7 +2503,6 @@ template <typename R, int TT, int MAX_THREADS = track_max_threads<R, TT>(), bool
 __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : track_min_ctas<R, TT>()))
     reed_track_kernel(const __grid_constant__ DevParams P, const __grid_constant__ DevBuf B, const int vt)
 {
-    static_assert(TT != REED_TT_NONE, "the ion-target-only model has its own kernel");
     extern __shared__ __align__(16) unsigned char smem[];
     Win<R, TT> W(smem, P.na, P.bond_cap, 0, P.g_nbins, P.act_cap,
                  B.spill ? B.spill + (size_t)blockIdx.x * B.spill_stride : nullptr);
@@ -2463,6 +2532,7 @@ __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : t
 
     int nbovf = 0, capovf = 0;
     unsigned triplets = 0;   // bond-angle terms of this thread in the current track
+    unsigned moved = 0;      // without lists: atoms that this thread has moved in it
     // phase clocks: the end of phases p .. PH_FORCE of a step (a later phase
     // overwrites its own; count_step adds them up), and whole laps outside
     auto mark = [&](int p) {
@@ -2604,6 +2674,10 @@ __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : t
             const R dt = R(S->dt), hdt = R(0.5) * R(S->dt);
             const int shift = S->shift;
             Partial<R> q = {R(0), R(0), R(0), R(0), R(0), R(0), 0, 0};
+            if constexpr (TT == REED_TT_NONE) {
+                moved += ion_block_pass<R, false>(P, B, H, W, dt, hdt, shift, q);
+                if (tid == 0 && shift) ++S->cnt[C_SHIFTS];
+            } else {
             // phase A: first half kick + drift of the atoms integrated before
             // the window moves, then the move (a step's kick and drift precede
             // its window update: an atom entering the integrated region is
@@ -2657,6 +2731,7 @@ __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : t
                 mark(PH_PASS1);
             }
             force_phase<R, TT, true>(P, H, W, hdt, q, false);
+            }
             reduce_partials<R, TT, false>(W, q);
             __syncthreads();
             if (lead && vt != (int)blockDim.x) {
@@ -2745,7 +2820,7 @@ __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : t
         // ---- track finished
         if (tid == 0) {
             S->t_mark = clock64();
-            count_listed<R>(S, S->ion.steps, S->ion.steps);
+            if constexpr (TT != REED_TT_NONE) count_listed<R>(S, S->ion.steps, S->ion.steps);
             S->cnt[C_STEPS] += (unsigned long long)(S->ion.steps - S->steps_from);
         }
         if (B.damage && lead) {
@@ -2763,6 +2838,10 @@ __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : t
             }
             finish_track<R>(P, B, S->ion, S->status);
             ++S->cnt[C_TRACKS];
+        }
+        if constexpr (TT == REED_TT_NONE) {
+            atomicAdd(&S->cnt[C_MOVED], (unsigned long long)moved);
+            moved = 0;
         }
         if constexpr (TT == REED_TT_TERSOFF) {
             const unsigned tr = __reduce_add_sync(0xffffffffu, triplets);

@@ -62,3 +62,56 @@ def test_density_of_atoms_without_a_force(R, O):
         ref, _ = O.trace(p, 11, t, steps)
         assert abs(ref[-1, 6] / ref[0, 6] - 1) > 1e-2
         np.testing.assert_allclose(traj[t, :, 4:7], ref[:, 4:7], rtol=1e-5, atol=0)
+
+
+def _sorted_run(R, w, n, **kw):
+    with R.Reed(w) as ctx:
+        ctx.run(n_ions=n, seed=7, record_capacity=20000, **kw)
+        rec = ctx.records()
+        st = ctx.stats()
+        damage = ctx.damage_map() if ctx.w["damage_n"] else None
+    return rec[np.argsort(rec["id"], kind="stable")], st, damage
+
+
+@pytest.mark.parametrize("threads", [128, 256])
+@pytest.mark.parametrize("name,over", [
+    ("b1kev_si_0k_zbl", dict(sigma=0.076, s_loc=0.2, damage_n=16)),
+    ("b1kev_si_0k_zbl", dict(n=2, sigma=0.076, rc=4.0, rt=3.5)),
+    ("b1kev_si_0k_zbl", dict(n=4, margin=1, sigma=0.076, spline_c=[0.1, -0.1, 0.2, 0.1, 0.0, -0.1])),
+    ("u85kev_uo2_300k_recoil", dict(n=3)),
+    ("kr85mev_uo2_300k_recoil", dict(n=3))])
+def test_a_block_follows_few_tracks(R, name, over, threads):
+    """A width of 128 or 256 puts a block of threads on each track while there
+    are two tracks per SM or fewer, and one warp beyond: the tracks are the same,
+    bit for bit (304 and 305 primaries: the two sides of the line on 152 SMs)."""
+    w = workload(name, thresholds=[], step_cap=500, **over)
+    rec, st, dam = _sorted_run(R, w, 304, threads=threads)
+    ref, st1, _ = _sorted_run(R, w, 305, threads=threads)
+    assert st["ctas_per_sm"] < st1["ctas_per_sm"]   # (a block each; one warp each)
+    assert rec.tobytes() == ref[:304].tobytes()
+    one, st0, _ = _sorted_run(R, w, 1, threads=threads, first_id=304)
+    assert one.tobytes() == ref[304:].tobytes()
+    for k in ("steps", "pair_evals", "atom_updates", "shifts", "stopped", "truncated", "backscattered"):
+        assert st[k] + st0[k] == st1[k], k
+    if dam is not None:   # (a map's sums: the order of 305 tracks' atomics)
+        with R.Reed(dict(w)) as ctx:
+            ctx.run(n_ions=304, seed=7, threads=64)
+            other = ctx.damage_map()   # another width: other roundings, the same tracks to statistics
+        assert abs(dam[0].sum() + dam[1] - other[0].sum() - other[1]) < 0.05 * (other[0].sum() + other[1])
+
+
+def test_a_block_makes_clones(R):
+    """Large windows leave room for few tracks per SM, and a width of 256 puts a
+    block on each there, cloning depths or not."""
+    w = workload("u85kev_uo2_300k_recoil", n=5, energy=2000.0, thresholds=[2.0, 5.0], step_cap=600)
+    rec, st, _ = _sorted_run(R, w, 60, threads=256)
+    assert st["ctas_per_sm"] * 256 <= 2048
+    assert st["clones"] > 60 and st["dropped_clones"] == 0 and st["tracks"] == 60 + st["clones"] == len(rec)
+    assert np.sum(np.ldexp(1.0, -rec["level"].astype(int))) == 60
+    again, _, _ = _sorted_run(R, w, 60, threads=256)
+    assert again.tobytes() == rec.tobytes()
+    # the part of each primary before its first depth, by one warp (one depth far off)
+    far = workload("u85kev_uo2_300k_recoil", n=3, energy=2000.0, thresholds=[1e6], step_cap=600)
+    a, sa, _ = _sorted_run(R, far, 20, threads=256)
+    b, sb, _ = _sorted_run(R, dict(far, thresholds=[]), 20, threads=256)
+    assert a.tobytes() == b.tobytes() and sa["ctas_per_sm"] != sb["ctas_per_sm"]
