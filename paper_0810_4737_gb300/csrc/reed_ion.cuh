@@ -338,10 +338,8 @@ __device__ __forceinline__ bool ion_move_atom(const HotParams<R>& H, IonWin<R>& 
     const R r2 = dist2(dx, dy, dz);
     const bool in = r2 < H.rc2;
     if (!in) {
-        if (t.x != R(0) || v.w != R(0)) {   // it has just left the cutoff
-            W.term[i] = {R(0), R(0), R(0), R(0)};
-            v.w = R(0);
-        }
+        if (t.x != R(0)) W.term[i] = {R(0), R(0), R(0), R(0)};   // it has just left the cutoff
+        v.w = R(0);
         if (act) vm = max(vm, dist2(v.x, v.y, v.z));
     }
     W.vel[i] = v;
