@@ -136,7 +136,13 @@ typedef struct {
     double thresholds[16];   /* ascending cloning depths d_1..d_k, A */
     double bin_width;        /* A (fixed by the first run after init/reset) */
     int64_t first_id;        /* id of the first primary of this run (ids are the RNG streams) */
-    int32_t threads_per_track; /* 0 = tuned or default, else 32/64/128/256 (512: pair-list model) */
+    /* Width of the sums over atoms, and with it the order in which they are
+     * added and a track's roundings: 0 = tuned or default (64 without target
+     * forces, else 256), else 32/64/128/256 (512: pair-list model).  The threads
+     * that follow a track are as many in an adjoint run, and without target
+     * forces at 128 or 256 in the mixed form while there are few tracks per SM;
+     * else one warp (no target forces), or 256 and more. */
+    int32_t threads_per_track;
     int32_t ctas_per_sm;       /* 0 = autotune / maximum occupancy */
     int32_t record_tracks;     /* 1: keep one reed_track_record per finished track */
     int32_t trace_tracks;      /* record the first trace_steps steps of primaries */
@@ -240,7 +246,10 @@ typedef struct {
                                 atom move, neighbour build, Tersoff pass 1, forces, track admin */
     double w_stopped, w_back, w_trunc;   /* weights */
     double kernel_ms;        /* device time of the last reed_run */
-    int32_t threads_per_track, ctas_per_sm, grid, smem_bytes;  /* last launch */
+    /* the last launch: width of the sums (see reed_run_opts; a CTA's own threads
+     * are chosen by the model and the number of tracks), tracks per SM at most,
+     * CTAs launched (a few Tersoff tracks: 2 or more CTAs on each), shared memory */
+    int32_t threads_per_track, ctas_per_sm, grid, smem_bytes;
     int64_t splits[16];      /* clones made on first passing cloning depth k+1 (the
                                 paper's per-depth split statistics, Sec. 3) */
     int64_t pooled;          /* clones run by another CTA than the one that made them

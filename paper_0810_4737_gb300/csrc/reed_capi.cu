@@ -1059,7 +1059,7 @@ int reed_stats(reed_ctx* ctx, reed_stats_t* out)
     out->kernel_ms = ctx->last_ms;
     out->threads_per_track = ctx->last_cfg.threads;
     out->ctas_per_sm = ctx->last_cfg.ctas_per_sm;
-    out->grid = ctx->last_cfg.grid;
+    out->grid = ctx->last_cfg.launched;
     out->smem_bytes = (int32_t)ctx->last_cfg.smem;
     return REED_OK;
 }
@@ -1762,7 +1762,7 @@ extern "C" int reed_run_static(const reed_lattice* lat, const reed_species* sp, 
         stats_out->w_trunc = w[W_TRUNC];
         stats_out->threads_per_track = L.threads;
         stats_out->ctas_per_sm = L.ctas_per_sm;
-        stats_out->grid = L.grid;
+        stats_out->grid = L.launched;
         stats_out->smem_bytes = (int32_t)L.smem;
     }
     if (status & ERR_NONFINITE) return fail(nullptr, REED_E_NONFINITE, "a track became non-finite");

@@ -70,3 +70,26 @@ def test_first_epoch_of_an_adaptive_run(R):
     rec, st, _ = _records(R, w, 50, 0, adaptive=True, n_initial=20, epoch_size=30, record_capacity=4000)
     assert st["primaries"] == 50
     assert rec[:20].tobytes() == ref.tobytes()
+
+
+@pytest.mark.parametrize("name,prec,thresholds,grids", [
+    # Tersoff: clusters of SMs on a few tracks, then a CTA for each, then two per SM
+    ("as10kev_si_300k_tersoff", 0, [], {1: (2, 4, 8), 31: (2, 4), 63: (2,), 64: (1,), 152: (1,), 304: (1,)}),
+    ("as10kev_si_300k_tersoff", 1, [], {1: (2, 4, 8), 31: (2, 4), 63: (2,), 64: (1,), 152: (1,)}),
+    ("ar30kev_ceo2_300k_buck", 0, [], {1: (1,), 152: (1,)}),
+    ("b1kev_si_0k_zbl", 0, [], {1: (1,), 153: (1,)}),
+    # with a cloning depth every CTA that fits is launched
+    ("as10kev_si_300k_tersoff", 0, [1e6], {5: None}),
+    ("b1kev_si_0k_zbl", 0, [1e6], {5: None})])
+def test_statistics_tell_the_ctas_launched(R, name, prec, thresholds, grids):
+    """(On 152 SMs, the count that the lines between the shapes are tested for.)"""
+    w = workload(name, thresholds=thresholds, step_cap=20)
+    for n, per_track in grids.items():
+        _, st, _ = _records(R, w, n, prec)
+        if per_track is None:
+            assert st["grid"] == 152 * st["ctas_per_sm"]
+        else:
+            assert st["grid"] % n == 0 and st["grid"] // n in per_track, (n, st["grid"])
+    if name.startswith("as10kev") and prec == 0 and not thresholds:
+        _, st, _ = _records(R, w, 305, prec)
+        assert st["grid"] == 304
