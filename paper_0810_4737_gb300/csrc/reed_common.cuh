@@ -19,7 +19,7 @@
 #define REED_MAX_THR 16
 #define REED_MAX_WARPS 24       // warps of a track's CTA at most (768 threads: one per atom of a 4^3-cell CeO2 window)
 #define REED_WIDE 512           // threads of a Tersoff track that has an SM to itself (mixed form)
-#define REED_MAX_TEAM 8         // CTAs that follow one Tersoff track together, at most
+#define REED_MAX_TEAM 4         // CTAs that follow one Tersoff track together, at most (see launch_tersoff)
 #define REED_POOL_SMS 256       // SMs whose busy tracks the clone pool counts apart
 #define REED_POOL_CTL (3 + REED_POOL_SMS)   // words of pool_ctl
 #define REED_ADJ_WARPS 8        // ... of an adjoint run

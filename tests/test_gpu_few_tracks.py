@@ -93,3 +93,11 @@ def test_statistics_tell_the_ctas_launched(R, name, prec, thresholds, grids):
     if name.startswith("as10kev") and prec == 0 and not thresholds:
         _, st, _ = _records(R, w, 305, prec)
         assert st["grid"] == 304
+
+
+def test_a_team_has_four_sms_at_most(R):
+    w = workload("as10kev_si_300k_tersoff", thresholds=[], step_cap=20)
+    for prec in (0, 1):
+        for n in (1, 7, 15, 31):
+            _, st, _ = _records(R, w, n, prec)
+            assert st["grid"] == 4 * n
