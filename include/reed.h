@@ -398,10 +398,14 @@ int reed_get_thresholds(reed_ctx* ctx, double* out16);
  * n_trial primaries of the given beam (ids from 2^40 up, so no primary of a
  * real run is repeated) once per candidate -- threads_per_track in {32, 64,
  * 128, 256, and 512 where the model allows it} and, for each, CTAs per SM
- * at the occupancy maximum, three quarters and half of it -- and keeps the
- * fastest (ion-steps per second of
+ * at the occupancy maximum, three quarters and half of it, where that changes
+ * the launch of n_trial tracks -- and keeps the fastest (ion-steps per second of
  * kernel time) for later runs of this context whose opt->threads_per_track
  * and opt->ctas_per_sm are 0 and whose precision and adjoint flag match opt.
+ * What is timed is the launch of n_trial tracks without cloning: give as many
+ * as a later run has, up to the number that fills the GPU (reed_stats: ctas_per_sm
+ * x SMs), since a run of fewer takes another shape.  threads_per_track is the
+ * width of the sums, so the choice decides the roundings of later tracks.
  * The trials run in a private context, so this context's tallies are not
  * touched; records, traces, damage and cloning are off in them, and
  * opt->step_cap bounds each trial track.  table (host, may be NULL) receives up

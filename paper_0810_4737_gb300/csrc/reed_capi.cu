@@ -7,6 +7,7 @@
 // the window in shared memory, grid = SMs x CTAs/SM) and runs it on the
 // caller's stream.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -1306,14 +1307,14 @@ int reed_autotune(reed_ctx* ctx, double ion_Z, double ion_M, double energy_eV, d
     double best = -1.0;
     static const int kThreads[5] = {32, 64, 128, 256, 512};
     for (int ti = 0; ti < 5; ++ti) {
-        // the occupancy maximum for this thread count: a run with ctas_per_sm
-        // far above it is clamped to it
+        // the occupancy maximum for this thread count and number of tracks: a run
+        // with ctas_per_sm far above it is clamped to it
         reed_run_opts probe = o;
         probe.threads_per_track = kThreads[ti];
         probe.ctas_per_sm = 1 << 20;
         probe.step_cap = 1;
         reed_reset(t);
-        rc = reed_run(t, ion_Z, ion_M, energy_eV, tilt_deg, rot_deg_lo, rot_deg_hi, 1, seed, &probe);
+        rc = reed_run(t, ion_Z, ion_M, energy_eV, tilt_deg, rot_deg_lo, rot_deg_hi, n_trial, seed, &probe);
         if (rc < 0) continue;   // does not fit (shared memory / threads)
         o.threads_per_track = kThreads[ti];
         const int occ = t->last_cfg.ctas_per_sm;
@@ -1323,6 +1324,9 @@ int reed_autotune(reed_ctx* ctx, double ion_Z, double ion_M, double energy_eV, d
             bool dup = false;
             for (int k = 0; k < ci; ++k) dup |= cands[k] == c;
             if (dup || c < 1) continue;
+            // (a trial without cloning has no more CTAs than tracks: below that,
+            // fewer per SM are the same launch)
+            if (ci > 0 && n_trial <= (int64_t)c * t->sms) continue;
             o.ctas_per_sm = c;
             reed_reset(t);
             rc = reed_run(t, ion_Z, ion_M, energy_eV, tilt_deg, rot_deg_lo, rot_deg_hi, n_trial, seed, &o);
@@ -1338,7 +1342,7 @@ int reed_autotune(reed_ctx* ctx, double ion_Z, double ion_M, double energy_eV, d
             if (v > best) {
                 best = v;
                 best_t = kThreads[ti];
-                best_c = c;
+                best_c = ci > 0 ? c : INT_MAX;   // (the maximum is no limit to a run of another shape)
             }
         }
     }
