@@ -160,7 +160,7 @@ template <typename R> __device__ __forceinline__ R regs_drag(const HotParams<R>&
     return H.gamma * (R(1) + H.s_loc * (I.rho * H.rho0_inv - R(1)));
 }
 
-// One half kick of the ion at the velocity it has (see ion_prologue).
+// One half kick of the ion at the velocity it has (see ion_step).
 template <typename R> __device__ __forceinline__ void regs_kick(const HotParams<R>& H, IonRegs<R>& I)
 {
     const R kd = regs_drag<R>(H, I);
@@ -173,7 +173,7 @@ template <typename R> __device__ __forceinline__ void regs_kick(const HotParams<
 }
 
 // Start of a step: dt, the ion's half kick and drift, window anchor check
-// (ion_prologue).  Returns whether the window moves; Aold is the anchor before.
+// (see ion_step).  Returns whether the window moves; Aold is the anchor before.
 template <typename R>
 __device__ __forceinline__ bool regs_prologue(const DevParams& P, const HotParams<R>& H, IonRegs<R>& I, int Aold[3],
                                               const double* thr, int nthr, int lane)
@@ -734,7 +734,7 @@ __device__ int follow_track(const DevParams& P, const DevBuf& B, const HotParams
         I.pmax = H.de_max > R(0) ? warp_max_pos(pm) : R(0);
         t0 = (unsigned)clock();
         c_force += t0 - t1;
-        // second half kick of the ion, end and cloning checks (ion_epilogue)
+        // second half kick of the ion, end and cloning checks (see ion_step)
         const bool on2 = I.rel[2] >= I.zsurf;
         regs_kick<R>(H, I);
         I.acc += lane == 3 ? (double)I.dt : 0.0;

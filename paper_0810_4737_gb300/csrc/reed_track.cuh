@@ -504,7 +504,6 @@ template <typename R> __device__ __forceinline__ bool is_second(const V4<R>& p) 
 template <typename R> __device__ __forceinline__ R of_species(const R q[2], const V4<R>& p) { return is_second(p) ? q[1] : q[0]; }
 
 // ---------------------------------------------------------------------------
-// ---------------------------------------------------------------------------
 // Target neighbour lists.  Rebuilt at track start, after a window move and
 // when the two longest atom paths since the last build add up to more than
 // the skin (a pair can then have closed in from beyond the list radius).
@@ -1727,8 +1726,8 @@ __device__ void force_phase(const DevParams& P, const HotParams<R>& H, Win<R, TT
     } else {
         // integrated atoms through their slots, then every other present atom
         const int nact = W.S->active_count;
-    #pragma unroll 1
-    for (int k = threadIdx.x; k < nact; k += blockDim.x)
+#pragma unroll 1
+        for (int k = threadIdx.x; k < nact; k += blockDim.x)
             atom_force<R, TT, KICK>(P, H, W, W.slot_atom[k], k, hdt, out, want_energy);
         if (KICK && !W.S->near_frozen) return;
         for (int i = threadIdx.x; i < P.na; i += blockDim.x) {
@@ -2204,7 +2203,6 @@ template <typename R> __device__ __forceinline__ bool may_reach(const HotParams<
     return !(dx * dx + dy * dy + dz * dz > H.rc2 * R(1.01));
 }
 
-// Copy the window (pos, vel, frc) between shared memory and a clone record.
 // ---------------------------------------------------------------------------
 // Shared clone pool (the paper's host handing returned clones to whichever
 // client is free, Sec. 3).  Lock-free: a slot is claimed with one CAS and no
@@ -2225,6 +2223,8 @@ __device__ __forceinline__ int pool_claim(const DevBuf& B, unsigned from, unsign
     return -1;
 }
 
+// Copy the window (pos, vel, frc) between shared memory and a clone record (_cg:
+// from a record that another SM may have written, through L2).
 template <typename R, int TT>
 __device__ __forceinline__ void copy_window_cg(const DevParams& P, Win<R, TT>& W, const unsigned char* rec)
 {
@@ -2489,16 +2489,16 @@ template <typename R, int TT> inline int track_threads(int act_cap)
 // arithmetic, are shared out, each result going into every CTA's window
 // through distributed shared memory.  CTA 0 leads: it alone takes tracks,
 // updates the ion, and tallies.  The others follow its decisions, so that all
-// pass the same cluster barriers.  61 As tracks in FP64, bound by the SMs' FP64
-// pipes: 361 -> 213 ms with teams of two; 37 in the mixed form (512 threads
-// alone on an SM: 46 ms; 256: 52 ms): 35 ms.
+// pass the same cluster barriers.  What it gives, for teams of 1, 2, 4 and 8:
+// see launch_tersoff.
 //
-// Much of a step's time is instruction fetch: the code of one step (centres 19
-// + 35 KB, ion 9 KB, lists) goes through the instruction cache once per step,
-// and a warp that runs alone waits for each line of it.  So the rare parts are
-// calls (REED_WINDOW), short loops are not unrolled, and the groups of 8 and 16
-// lanes share their code: 4096 As ions of 10 keV 1139 -> 977 ms, and 823 ms with
-// the counters out of the ion update (see ion_step).
+// Much of a step's time is instruction fetch: the code of one step (centres,
+// ion, lists) goes through the instruction cache once per step, and a warp that
+// runs alone waits for each line of it (0.9 stalls per issued instruction; 1.8
+// with everything inlined and unrolled).  So the rare parts are calls
+// (REED_WINDOW), short loops are not unrolled, and the groups of 8 and 16 lanes
+// share their code: 4096 As ions of 10 keV 1139 -> 977 ms, and 816 ms with the
+// counters out of the ion update (see ion_step).
 template <typename R, int TT, int MAX_THREADS = track_max_threads<R, TT>(), bool TEAM = false>
 __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : track_min_ctas<R, TT>()))
     reed_track_kernel(const __grid_constant__ DevParams P, const __grid_constant__ DevBuf B, const int vt)
