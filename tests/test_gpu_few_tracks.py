@@ -101,3 +101,20 @@ def test_a_team_has_four_sms_at_most(R):
         for n in (1, 7, 15, 31):
             _, st, _ = _records(R, w, n, prec)
             assert st["grid"] == 4 * n
+
+
+@pytest.mark.parametrize("n,margin,prec,team", [
+    (2, 0, 0, False), (3, 0, 0, False), (3, 1, 0, False), (4, 1, 0, False), (5, 2, 0, False), (5, 1, 0, True),
+    (6, 1, 0, True), (3, 0, 1, True), (4, 1, 1, False), (5, 1, 1, True)])
+def test_teams_where_there_are_many_centres(R, n, margin, prec, team):
+    """Small windows, and in the mixed form windows without a frozen layer, get no
+    teams; the tracks are those of the batch launch (which a cloning depth out of
+    reach selects) in every shape."""
+    w = workload("as10kev_si_300k_tersoff", n=n, margin=margin, thresholds=[], energy=300.0, step_cap=120 if prec else 300)
+    rec, st, _ = _records(R, w, 7, prec)
+    assert st["grid"] == (28 if team else 7)
+    ref, st1, _ = _records(R, dict(w, thresholds=[1e6]), 7, prec)
+    assert st1["grid"] % 152 == 0
+    assert rec.tobytes() == ref.tobytes()
+    for k in ("steps", "pair_evals", "bond_evals", "triplets", "atom_updates", "shifts"):
+        assert st[k] == st1[k], k
