@@ -431,11 +431,12 @@ int launch_shape(reed_ctx* ctx, DevParams& P, bool f64, size_t optin, int device
     auto fit = [&](int cap) {   // tracks per SM with `cap` rows
         P.bond_cap = cap;
         L.smem = bytes(cap);
-        return f64 ? reed_f64::occupancy(tt, L.threads, L.smem, occ, P.adjoint, P.act_cap, L.block)
-                   : reed_f32::occupancy(tt, L.threads, L.smem, occ, P.adjoint, P.act_cap, L.block);
+        return f64 ? reed_f64::occupancy(tt, L.threads, L.smem, occ, P.adjoint, P.act_cap, L.block, L.narrow)
+                   : reed_f32::occupancy(tt, L.threads, L.smem, occ, P.adjoint, P.act_cap, L.block, L.narrow);
     };
     P.refresh_cap = base;
     L.block = false;
+    L.narrow = 0;
     if (bytes(base) > optin)
         return fail(ctx, REED_E_SMEM, "window of %d atoms needs %zu B of shared memory (max %zu)", P.na, bytes(base), optin);
     CK(fit(base));
@@ -447,6 +448,25 @@ int launch_shape(reed_ctx* ctx, DevParams& P, bool f64, size_t optin, int device
         L.block = false;
         CK(fit(base));
         return REED_OK;
+    }
+    // In the FP64 form a track with target forces takes the registers of 256
+    // threads or more, and in small windows an SM has the shared memory for more
+    // tracks than that.  A narrower width gets a CTA of as many threads (64 at
+    // least: the second warp keeps the counters; and one for every two integrated
+    // atoms) when more tracks fit then and there are more than the wider CTAs
+    // hold.  310 and 1000 tracks, wide -> narrow, ms: As, 8 integrated atoms in 3^3
+    // cells, width 128: 35.3 -> 19.9, 106 -> 62.8; 64 in 4^3, width 64: 59.0 -> 52.9,
+    // 143 -> 117; Ar, 12 in 3^3, width 64: 43.0 -> 22.5, 90 -> 52.5.  216 in 3^3: 128
+    // threads 75.9 -> 71.7, but 64 threads 94.8.
+    const int narrow = std::max(std::max(L.threads, 64), (P.act_cap / 2 + 31) / 32 * 32);
+    if (f64 && tt != REED_TT_NONE && narrow <= 128 && (P.nthr > 0 || P.n_primaries > (int64_t)L.sms * *occ)) {
+        const int wide = *occ;
+        L.narrow = narrow;
+        CK(fit(base));
+        if (*occ <= wide) {
+            L.narrow = 0;
+            CK(fit(base));
+        }
     }
     const int tracks = *occ;
     if (tt != REED_TT_TERSOFF || base >= P.na || tracks < 1) return REED_OK;
