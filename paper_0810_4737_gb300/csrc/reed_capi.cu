@@ -406,8 +406,13 @@ int neighbor_error(reed_ctx* ctx, const unsigned long long* c)
 // U in 4^3 18.8 -> 19.3; width 128: 2400 B in 6^3 (2 and 2) 46.9 -> 49.0; width 64:
 // 300 B in 3^3 2.58 -> 3.38.  The FP64 form is bound by its pipe, and one warp is
 // the faster one from 3^3 cells on (300 B, width 256: 3.53 -> 4.48).
+//   An adjoint run has a CTA of its width either way, for its reverse pass; at 128
+// and 256 all of it takes the forward steps too, at any number of tracks: B of 5
+// keV, one warp -> block, width 256, 16 tracks 57.9 -> 41.0 ms and 2000 tracks 240
+// -> 177, width 128 53.2 -> 47.0 and 132 -> 121 (width 64, one warp: 51.1 and 113).
 bool ion_by_block(const DevParams& P, int threads, int sms, int warps, int blocks)
 {
+    if (P.adjoint) return true;
     if (warps <= 3) return threads == 256 || blocks > warps;
     return P.nthr == 0 && P.n_primaries <= 2 * (int64_t)sms;
 }
@@ -440,7 +445,7 @@ int launch_shape(reed_ctx* ctx, DevParams& P, bool f64, size_t optin, int device
     if (bytes(base) > optin)
         return fail(ctx, REED_E_SMEM, "window of %d atoms needs %zu B of shared memory (max %zu)", P.na, bytes(base), optin);
     CK(fit(base));
-    if (tt == REED_TT_NONE && !P.adjoint && !f64 && (L.threads == 128 || L.threads == 256)) {
+    if (tt == REED_TT_NONE && !f64 && (L.threads == 128 || L.threads == 256)) {
         const int warps = *occ;
         L.block = true;
         CK(fit(base));

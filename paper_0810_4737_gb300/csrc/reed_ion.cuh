@@ -1,5 +1,6 @@
 // reed_ion.cuh -- the track stepper of the ion-target-only model (target
-// model NONE): one warp follows one track.
+// model NONE): one warp follows one track.  (Wide runs that would leave an SM's
+// warps idle get a block of threads per track, see ion_by_block.)
 //
 // Without target-target forces an atom that the ion has not come near is at
 // rest and stays at rest, so a step concerns three sets only:
@@ -22,14 +23,15 @@
 // the groups of 32 in order -- the summation order of a block of vt threads
 // with one atom per thread and pass.  threads_per_track selects vt.
 //
-// What bounds a step: instruction issue and its latency -- about 830 warp
-// instructions and 4300 cycles in the mixed form when a track runs alone --
-// and in the FP64 form the FP64 pipe (63 % busy, 308 instructions a step).  A
-// block of 64 threads that tested every atom of the window in each step,
-// with one thread's ion update between two barriers, took 1700 instructions
-// and 6200 cycles.  Measured on whole runs (block of 64 -> one warp): 32 B
-// ions of 1 keV 19.1 -> 13.2 ms, 3001 of 10 keV 218 -> 123 ms, 500 of 1 keV in
-// FP64 311 -> 140 ms, 131 Kr of 85 MeV (10^4 steps each) 50.9 -> 31.1 ms.
+// What bounds a step: instruction issue and its latency -- some 850 warp
+// instructions, 4200 cycles in the mixed form when a track runs alone and 5200
+// with 16 on an SM, whose issue slots are then 62 % busy -- and in the FP64 form
+// the FP64 pipe (64 % busy with four tracks on an SM).  A block of 64 threads that
+// tested every atom of the window in each step, with one thread's ion update
+// between two barriers, took 1700 instructions.  Measured on whole runs (block
+// of 64 -> one warp): 32 B ions of 1 keV 17.3 -> 11.8 ms, 3001 of 10 keV 200 -> 114
+// ms, 500 of 1 keV in FP64 300 -> 98 ms, 131 Kr of 85 MeV (10^4 steps each) 51.1
+// -> 27.2 ms.
 #pragma once
 
 #include <type_traits>
@@ -810,7 +812,8 @@ __device__ int follow_track(const DevParams& P, const DevBuf& B, const HotParams
 // The persistent kernel of the ion-target-only model: one track per CTA.
 // Without the adjoint a CTA is one warp.  With it (ADJ) a CTA has vt threads:
 // the first warp follows the track, all of them run the reverse pass of the
-// truncated-segment adjoint.
+// truncated-segment adjoint.  (Where a block of threads follows a track, with the
+// adjoint or without: reed_track_kernel.)
 template <typename R, bool ADJ>
 __global__ void __launch_bounds__(ADJ ? 256 : 32, (ADJ ? (sizeof(R) == 4 ? 2 : 1) : (sizeof(R) == 4 ? 16 : 10)))
     reed_ion_kernel(const __grid_constant__ DevParams P, const __grid_constant__ DevBuf B, const int vt)
@@ -869,17 +872,8 @@ __global__ void __launch_bounds__(ADJ ? 256 : 32, (ADJ ? (sizeof(R) == 4 ? 2 : 1
         if (!ADJ) __syncwarp();   // (lane 0 goes on to write the next track's; an adjoint run ends on a barrier)
         if (src == SRC_NONE) break;
         if constexpr (ADJ) {
-            // truncated-segment sensitivities of the final depth
-            if (adjbase && B.grads && S->rec_index >= 0) {
-                double g[REED_NTHETA] = {0, 0, 0, 0, 0, 0, 0, 0};
-                if (S->status == REED_TRACK_STOPPED) {
-                    Win<R, REED_TT_NONE> WA(smem, P.na, 0, 1);
-                    AdjScratch<R, REED_TT_NONE> A(adjbase, P, B.entry_bytes);
-                    adjoint_track<R, REED_TT_NONE>(P, H, WA, A, g);
-                }
-                if (tid == 0)
-                    for (int k = 0; k < REED_NTHETA; ++k) B.grads[(size_t)S->rec_index * REED_NTHETA + k] = g[k];
-            }
+            Win<R, REED_TT_NONE> WA(smem, P.na, 0, 1);
+            adjoint_gradient<R>(P, B, H, WA, adjbase);
             __syncthreads();
         }
     }

@@ -33,7 +33,17 @@
 enum { SRC_NONE = 0, SRC_PRIMARY = 1, SRC_CLONE = 2, SRC_STOLEN = 3 };
 enum { POOL_EMPTY = 0, POOL_WRITING = 1, POOL_FULL = 2, POOL_READING = 3 };
 
-enum { EV_NONE = 0, EV_END = 1, EV_CLONE = 2 };
+enum { EV_NONE = 0, EV_END = 1, EV_CLONE = 2, EV_SAVE = 3 };
+
+enum { REED_NTHETA = 8 };
+#define REED_STEP_RING 256
+
+// Frozen quantities of one step.
+template <typename R> struct StepRec {
+    R dt;
+    int A[3];    // anchor after the step
+    int flags;   // bit 0: drag on at the first half kick, bit 1: at the second, bit 2: window moved
+};
 
 // counters a CTA of the ion-target-only model keeps in shared memory
 enum {
@@ -2029,8 +2039,9 @@ __device__ __noinline__ void trace_step(const DevParams& P, const DevBuf& B, con
 // cloning checks of the step (not with BEGIN, the start of a track), then the
 // next step's dt from the fastest particle, first half kick, drift and window
 // anchor check (Fig. "moving cell": the main cell follows the ion).  Returns
-// EV_NONE / EV_END / EV_CLONE (no next step prepared); sets S->event,
-// S->status and S->nclone.
+// EV_NONE / EV_END / EV_CLONE / EV_SAVE (no next step prepared); sets S->event,
+// S->status and S->nclone.  ADJ: writes the step's frozen quantities to `ring`
+// and asks for a checkpoint (EV_SAVE) every adj_every steps.
 //
 // The rest of the CTA waits here, so what counts is the length of the chain.
 // Lanes 0-2 hold one component each and lane 3 the time: an FP64 addition
@@ -2040,9 +2051,9 @@ __device__ __noinline__ void trace_step(const DevParams& P, const DevBuf& B, con
 // thread with rolled loops: 4.0k).
 // `rows` warps left partial sums; those of the ion (columns 0-3) are in `vrows`
 // rows.
-template <typename R, bool BEGIN>
+template <typename R, bool BEGIN, bool ADJ = false>
 __device__ __forceinline__ int ion_step(const DevParams& P, const DevBuf& B, const HotParams<R>& H, TrackShared<R>* S,
-                                        int rows, int vrows, bool tracing)
+                                        int rows, int vrows, bool tracing, StepRec<R>* ring = nullptr)
 {
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, c = min(lane, 2);
@@ -2103,6 +2114,22 @@ __device__ __forceinline__ int ion_step(const DevParams& P, const DevBuf& B, con
             __syncwarp();
             trace_step<R>(P, B, S, x, v);
         }
+        if constexpr (ADJ) {
+            // (the drag is on at both half kicks of a step that begin on the same side:
+            // the second of one step and the first of the next see the same depth)
+            const bool on = relz >= zsurf;
+            if (lane == 0) {
+                StepRec<R> sr;
+                sr.dt = dt;
+                sr.A[0] = I.A[0];
+                sr.A[1] = I.A[1];
+                sr.A[2] = I.A[2];
+                sr.flags = (S->on1 ? 1 : 0) | (on ? 2 : 0) | (S->shift ? 4 : 0);
+                ring[(steps - 1) % REED_STEP_RING] = sr;
+                S->on1 = on;
+            }
+            if (ev == EV_NONE && steps % P.adj_every == 0) ev = EV_SAVE;
+        }
         if (REED_RARE(ev == EV_NONE && relz >= S->zthr)) {
             if (lane < 3) I.x[lane] = x;
             __syncwarp();
@@ -2110,6 +2137,9 @@ __device__ __forceinline__ int ion_step(const DevParams& P, const DevBuf& B, con
             if (lane == 0) S->nclone = nc;
             if (nc) ev = EV_CLONE;
         }
+    }
+    if constexpr (ADJ && BEGIN) {
+        if (lane == 0) S->on1 = relz >= zsurf;
     }
     bool moved = false;
     if (ev == EV_NONE) {
@@ -2175,10 +2205,10 @@ template <typename R> __device__ __forceinline__ void count_step(TrackShared<R>*
     __syncwarp();
     if (lane == 0) S->mark[0] = S->mark[PH_FORCE + 1];
 }
-template <typename R>
+template <typename R, bool ADJ>
 __device__ __noinline__ void ion_begin(const DevParams& P, const DevBuf& B, TrackShared<R>* S)
 {
-    ion_step<R, true>(P, B, hot<R>(P), S, 0, 0, false);
+    ion_step<R, true, ADJ>(P, B, hot<R>(P), S, 0, 0, false);
 }
 
 // Work counters that follow from the list sizes, brought up to date before the
@@ -2499,16 +2529,26 @@ template <typename R, int TT> inline int track_threads(int act_cap)
 // (REED_WINDOW), short loops are not unrolled, and the groups of 8 and 16 lanes
 // share their code: 4096 As ions of 10 keV 1139 -> 977 ms, and 816 ms with the
 // counters out of the ion update (see ion_step).
-template <typename R, int TT, int MAX_THREADS = track_max_threads<R, TT>(), bool TEAM = false>
-__global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : track_min_ctas<R, TT>()))
+// ADJ (ion-target-only model): the adjoint's checkpoints and step records while
+// the track runs, and its reverse pass at the end (see reed_ion_kernel).
+template <typename R, int TT, int MAX_THREADS = track_max_threads<R, TT>(), bool TEAM = false, bool ADJ = false>
+__global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : (ADJ ? 2 : track_min_ctas<R, TT>())))
     reed_track_kernel(const __grid_constant__ DevParams P, const __grid_constant__ DevBuf B, const int vt)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    Win<R, TT> W(smem, P.na, P.bond_cap, 0, P.g_nbins, P.act_cap,
+    static_assert(!ADJ || (TT == REED_TT_NONE && !TEAM), "the adjoint runs without target-target forces");
+    Win<R, TT> W(smem, P.na, P.bond_cap, ADJ, P.g_nbins, P.act_cap,
                  B.spill ? B.spill + (size_t)blockIdx.x * B.spill_stride : nullptr);
     TrackShared<R>* S = W.S;
     const HotParams<R>& H = hot<R>(P);
     const int tid = threadIdx.x;
+    unsigned char* adjbase = ADJ ? B.adj + (size_t)blockIdx.x * B.adj_stride : nullptr;
+    auto checkpoint = [&](long long step) {
+        if constexpr (ADJ) {
+            save_state<R, TT>(P, W, adjbase + (size_t)((step / P.adj_every) % P.adj_nck) * B.entry_bytes);
+            __syncthreads();
+        }
+    };
     if (TEAM) {
         W.team = cluster_size();
         W.rank = cluster_rank();
@@ -2655,6 +2695,7 @@ __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : t
             capovf += n.y;
             if (lead) triplets += (unsigned)n.z;   // (of a team, counted by the leader)
         }
+        checkpoint(0);
         const bool tracing = (src == SRC_PRIMARY) && (S->pidx < P.trace_tracks);
 
         // ---- step loop
@@ -2666,7 +2707,7 @@ __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : t
         bool need_prologue = true;
         for (;;) {
             if (need_prologue) {
-                if (lead && tid < 32) ion_begin<R>(P, B, S);
+                if (lead && tid < 32) ion_begin<R, ADJ>(P, B, S);
                 team_sync();
                 follow();
             }
@@ -2739,7 +2780,10 @@ __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : t
                 __syncthreads();
             }
             mark(PH_FORCE);
-            if (lead && tid < 32) ion_step<R, false>(P, B, H, S, (int)blockDim.x >> 5, vt >> 5, tracing);
+            if (lead && tid < 32)
+                ion_step<R, false, ADJ>(P, B, H, S, (int)blockDim.x >> 5, vt >> 5, tracing,
+                                        ADJ ? reinterpret_cast<StepRec<R>*>(adjbase + (size_t)P.adj_nck * B.entry_bytes)
+                                            : nullptr);
             else if (lead && tid < 64) count_step<R>(S, (int)blockDim.x >> 5);
             team_sync();
             follow();
@@ -2750,6 +2794,10 @@ __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : t
             }
             need_prologue = true;
             if (ev == EV_END) break;
+            if (ADJ && ev == EV_SAVE) {
+                checkpoint(S->ion.steps);
+                continue;
+            }
             // ---- cloning (Sec. 2): push one record per level passed
             const int nc = S->nclone;
             __syncthreads();
@@ -2836,8 +2884,13 @@ __global__ void __launch_bounds__(MAX_THREADS, (MAX_THREADS == REED_WIDE ? 1 : t
                 ++S->cnt[C_FAILED];
                 atomicOr(B.status, ERR_NONFINITE);
             }
-            finish_track<R>(P, B, S->ion, S->status);
+            const long long k = finish_track<R>(P, B, S->ion, S->status);
+            if constexpr (ADJ) S->rec_index = k;
             ++S->cnt[C_TRACKS];
+        }
+        if constexpr (ADJ) {
+            __syncthreads();
+            adjoint_gradient<R>(P, B, H, W, adjbase);
         }
         if constexpr (TT == REED_TT_NONE) {
             atomicAdd(&S->cnt[C_MOVED], (unsigned long long)moved);

@@ -187,3 +187,41 @@ def test_full_size_sensitivities_are_finite_and_deterministic(R):
     assert np.array_equal(out[0][1][o0], out[1][1][o1])
     np.testing.assert_allclose(out[0][2], out[1][2], rtol=1e-12, atol=1e-18)
     np.testing.assert_allclose(out[0][3], out[1][3], rtol=1e-9, atol=1e-12 * np.max(np.abs(gt)))
+
+
+@pytest.mark.parametrize("threads", [128, 256])
+@pytest.mark.parametrize("seg,every", [(220, 20), (60, 10)])
+def test_block_form_against_oracle(R, O, threads, seg, every):
+    """Widths of 128 and 256 run the mixed form's adjoint with a block of threads
+    per track, the forward part too.  The tracks are those of a run without the
+    adjoint, bit for bit; the sensitivities of short tracks are held to 3e-3 of the
+    oracle's: the roundings of the test above in another order of sums, three
+    times its bound."""
+    w = workload("b10kev_si_300k_adjoint", energy=1000.0, e_stop=900.0, **THETA["shifted"])
+    n = 24
+    rec, g = _gpu(R, w, n, 0, adj_segment=seg, adj_every=every, threads=threads)
+    with R.Reed(w) as ctx:
+        ctx.run(n_ions=n, seed=0, threads=threads)
+        plain = ctx.records()
+    assert np.sort(rec, order="id").tobytes() == np.sort(plain, order="id").tobytes()
+    stopped = np.nonzero(rec["status"] == STOPPED)[0]
+    refs = _oracle_tangents(O, O.params(w), 0, rec["primary"][stopped], seg, every)
+    compared = 0
+    for i, ref in zip(stopped, refs):
+        if ref["T"] != rec["steps"][i] or abs(ref["z"] - rec["z"][i]) > 1e-3:
+            continue
+        compared += 1
+        scale = np.maximum(np.abs(ref["grad"]), 1e-3 * np.max(np.abs(ref["grad"])))
+        assert np.max(np.abs(g[i] - ref["grad"]) / scale) <= 3e-3, (i, g[i], ref["grad"])
+    assert compared >= len(stopped) - len(stopped) // 8
+
+
+def test_block_form_of_whole_tracks(R):
+    """Whole tracks with window moves and many checkpoints, more than the block
+    form has CTAs: repeatable, and the same whichever CTA runs them."""
+    w = workload("b10kev_si_300k_adjoint", energy=500.0, s_loc=0.1)
+    rec, g = _gpu(R, w, 700, 0, seed=9, threads=256)
+    few, gf = _gpu(R, w, 9, 0, seed=9, threads=256)
+    a, b = np.argsort(rec["id"]), np.argsort(few["id"])
+    assert rec[a][:9].tobytes() == few[b].tobytes() and g[a][:9].tobytes() == gf[b].tobytes()
+    assert (np.abs(g[rec["status"] == STOPPED]).max(axis=1) > 0).all()
