@@ -395,17 +395,19 @@ int neighbor_error(reed_ctx* ctx, const unsigned long long* c)
 // Whether a block of `threads` threads follows a track of the ion-target-only
 // model (mixed form), and not one warp; warps, blocks: how many tracks an SM
 // holds either way.  A block takes a step sooner and more of an SM: it is taken
-// where a width of 128 or 256 is asked for and warps would be idle, with two
-// tracks per SM or fewer, or in a window so large that an SM's shared memory
-// holds three tracks or fewer (at a width of 128 only if it holds more blocks:
-// their windows need no list).  Measured, one warp -> block, 1200 steps: width
-// 256, 300 tracks: B in 3^3 cells of Si 3.24 -> 2.30 ms, U in 3^3 of UO2 3.99 ->
-// 2.78; 2400 tracks, U in 5^3 49.7 -> 26.1, in 6^3 129.6 -> 81.3.  Width 128, 300
-// tracks: 2.81 -> 2.60 and 3.56 -> 3.03; 2400 U in 5^3 (2 warps, 3 blocks) 46.2 ->
-// 34.9.  On the other side of the line, width 256: 600 B in 3^3 3.26 -> 4.52, 2400
-// U in 4^3 18.8 -> 19.3; width 128: 2400 B in 6^3 (2 and 2) 46.9 -> 49.0; width 64:
-// 300 B in 3^3 2.58 -> 3.38.  The FP64 form is bound by its pipe, and one warp is
-// the faster one from 3^3 cells on (300 B, width 256: 3.53 -> 4.48).
+// where a width of 128 or 256 is asked for and warps would be idle, while all
+// tracks are followed at once (256; counting one more per cloning depth) or there
+// are two per SM or fewer (128, without cloning), or in a window so large that an
+// SM's shared memory holds three tracks or fewer (at a width of 128 only if it
+// holds more blocks: their windows need no list).  Measured, one warp -> block, 1200
+// steps: width 256, 300 tracks: B in 3^3 cells of Si 3.24 -> 2.30 ms, U in 3^3 of
+// UO2 3.99 -> 2.78; 2400 tracks, U in 5^3 49.7 -> 26.1, in 6^3 129.6 -> 81.3.  Width
+// 128, 300 tracks: 2.81 -> 2.60 and 3.56 -> 3.03; 2400 U in 5^3 (2 warps, 3 blocks)
+// 46.2 -> 34.9.  On the other side of the line, width 256: 600 B in 3^3 3.26 ->
+// 4.52, 2400 U in 4^3 18.8 -> 19.3; width 128: 600 B in 5^3 4.64 -> 5.00, 2400 in 6^3
+// (2 and 2) 46.9 -> 49.0, 4 Kr with 8 cloning distances 7.34 -> 7.98; width 64: 300 B in 3^3 2.58 -> 3.38.  The FP64 form is
+// bound by its pipe, and one warp is the faster one from 3^3 cells on (300 B,
+// width 256: 3.53 -> 4.48).
 //   An adjoint run has a CTA of its width either way, for its reverse pass; at 128
 // and 256 all of it takes the forward steps too, at any number of tracks: B of 5
 // keV, one warp -> block, width 256, 16 tracks 57.9 -> 41.0 ms and 2000 tracks 240
@@ -414,7 +416,8 @@ bool ion_by_block(const DevParams& P, int threads, int sms, int warps, int block
 {
     if (P.adjoint) return true;
     if (warps <= 3) return threads == 256 || blocks > warps;
-    return P.nthr == 0 && P.n_primaries <= 2 * (int64_t)sms;
+    if (threads == 128 && P.nthr > 0) return false;
+    return P.n_primaries * (1 + P.nthr) <= (int64_t)(threads == 256 ? blocks : 2) * sms;
 }
 
 // The launch shape of a run: shared memory, tracks per SM and the rows of the

@@ -82,20 +82,22 @@ def _sorted_run(R, w, n, **kw):
     ("kr85mev_uo2_300k_recoil", dict(n=3))])
 def test_a_block_follows_few_tracks(R, name, over, threads):
     """A width of 128 or 256 puts a block of threads on each track while there
-    are two tracks per SM or fewer, and one warp beyond: the tracks are the same,
-    bit for bit (304 and 305 primaries: the two sides of the line on 152 SMs)."""
+    are two tracks per SM (128) or all run at once (256: three blocks per SM),
+    and one warp beyond: the tracks are the same, bit for bit, on the two sides of
+    the line on 152 SMs."""
     w = workload(name, thresholds=[], step_cap=500, **over)
-    rec, st, dam = _sorted_run(R, w, 304, threads=threads)
-    ref, st1, _ = _sorted_run(R, w, 305, threads=threads)
+    line = 304 if threads == 128 else 456
+    rec, st, dam = _sorted_run(R, w, line, threads=threads)
+    ref, st1, _ = _sorted_run(R, w, line + 1, threads=threads)
     assert st["ctas_per_sm"] < st1["ctas_per_sm"]   # (a block each; one warp each)
-    assert rec.tobytes() == ref[:304].tobytes()
-    one, st0, _ = _sorted_run(R, w, 1, threads=threads, first_id=304)
-    assert one.tobytes() == ref[304:].tobytes()
+    assert rec.tobytes() == ref[:line].tobytes()
+    one, st0, _ = _sorted_run(R, w, 1, threads=threads, first_id=line)
+    assert one.tobytes() == ref[line:].tobytes()
     for k in ("steps", "pair_evals", "atom_updates", "shifts", "stopped", "truncated", "backscattered"):
         assert st[k] + st0[k] == st1[k], k
-    if dam is not None:   # (a map's sums: the order of 305 tracks' atomics)
+    if dam is not None:
         with R.Reed(dict(w)) as ctx:
-            ctx.run(n_ions=304, seed=7, threads=64)
+            ctx.run(n_ions=line, seed=7, threads=64)
             other = ctx.damage_map()   # another width: other roundings, the same tracks to statistics
         assert abs(dam[0].sum() + dam[1] - other[0].sum() - other[1]) < 0.05 * (other[0].sum() + other[1])
 
@@ -110,8 +112,9 @@ def test_a_block_makes_clones(R):
     assert np.sum(np.ldexp(1.0, -rec["level"].astype(int))) == 60
     again, _, _ = _sorted_run(R, w, 60, threads=256)
     assert again.tobytes() == rec.tobytes()
-    # the part of each primary before its first depth, by one warp (one depth far off)
-    far = workload("u85kev_uo2_300k_recoil", n=3, energy=2000.0, thresholds=[1e6], step_cap=600)
-    a, sa, _ = _sorted_run(R, far, 20, threads=256)
-    b, sb, _ = _sorted_run(R, dict(far, thresholds=[]), 20, threads=256)
-    assert a.tobytes() == b.tobytes() and sa["ctas_per_sm"] != sb["ctas_per_sm"]
+    # a few primaries with cloning depths by blocks, and among many by one warp each
+    w = workload("u85kev_uo2_300k_recoil", n=3, energy=2000.0, thresholds=[2.0, 5.0], step_cap=600)
+    a, sa, _ = _sorted_run(R, w, 20, threads=256)
+    b, sb, _ = _sorted_run(R, w, 200, threads=256)
+    assert sa["ctas_per_sm"] < sb["ctas_per_sm"] and sa["clones"] > 20
+    assert a.tobytes() == b[b["primary"] < 20].tobytes()
