@@ -138,10 +138,12 @@ typedef struct {
     int64_t first_id;        /* id of the first primary of this run (ids are the RNG streams) */
     /* Width of the sums over atoms, and with it the order in which they are
      * added and a track's roundings: 0 = tuned or default (64 without target
-     * forces, else 256), else 32/64/128/256 (512: pair-list model).  The threads
-     * that follow a track are as many in an adjoint run, and without target
-     * forces at 128 or 256 in the mixed form while there are few tracks per SM;
-     * else one warp (no target forces), or 256 and more. */
+     * forces, else 256), else 32/64/128/256 (512: pair-list model).  How many
+     * threads follow a track is the library's choice: without target forces one
+     * warp, or as many threads as the width in an adjoint run and where a width
+     * of 128 or 256 would leave an SM's warps idle; with target forces 256 or
+     * more, or fewer in FP64 runs of a narrower width.  A track's result does
+     * not depend on it. */
     int32_t threads_per_track;
     int32_t ctas_per_sm;       /* 0 = autotune / maximum occupancy */
     int32_t record_tracks;     /* 1: keep one reed_track_record per finished track */
@@ -239,7 +241,9 @@ typedef struct {
     int64_t stopped, backscattered, truncated, failed;
     int64_t dropped_clones;  /* clones lost to a full stack */
     int64_t nb_overflow;     /* neighbour-list entries that found no room (REED_E_NEIGHBOR) */
-    int64_t bond_cap_overflow; /* needed atoms left without a list row (REED_E_NEIGHBOR) */
+    int64_t bond_cap_overflow; /* needed atoms left without a list row (REED_E_NEIGHBOR; the table has
+                                  the rows of a perfect window, a quarter more, and what the shared
+                                  memory of the launch leaves) */
     int64_t triplets;        /* Tersoff bond-angle (zeta) terms evaluated */
     int64_t atom_updates;    /* integrated target-atom updates (atoms x steps) */
     int64_t phase_cycles[6]; /* SM clock cycles per step phase, summed over CTAs: ion update,
