@@ -417,7 +417,7 @@ bool ion_by_block(const DevParams& P, int threads, int sms, int warps, int block
     if (P.adjoint) return true;
     if (warps <= 3) return threads == 256 || blocks > warps;
     if (threads == 128 && P.nthr > 0) return false;
-    return P.n_primaries * (1 + P.nthr) <= (int64_t)(threads == 256 ? blocks : 2) * sms;
+    return P.n_primaries <= (int64_t)(threads == 256 ? blocks : 2) * sms / (1 + P.nthr);
 }
 
 // The launch shape of a run: shared memory, tracks per SM and the rows of the
